@@ -87,9 +87,10 @@ typedef enum {
      * positions and momenta (Boris-tan excepted: tan is not correctly rounded). */
     FETDPIC_FP64 = 0,
     /* FP32 gather/push/deposit with cell-local barycentric positions and
-     * momenta in units of c; FP64 for the Lorentz factor and momentum update
-     * of particles with gamma > 10, for the field unknowns e, b, the Faraday
-     * update, C^T [*mu^-1] b - i and the checks.  The SPAI product dt M r of
+     * momenta in units of c; double-float (48 bits; FP64 beyond its range) for
+     * the Lorentz factor and momentum update of particles with gamma > 10;
+     * FP64 for the field unknowns e, b, the Faraday update, C^T [*mu^-1] b - i
+     * and the checks.  The SPAI product dt M r of
      * the Ampere update runs in FP32 (FP32 matrix values, r rounded to FP32,
      * FP32 sums) and is added to the FP64 e. */
     FETDPIC_FP32 = 1

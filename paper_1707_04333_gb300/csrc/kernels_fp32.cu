@@ -1,8 +1,8 @@
 // FP32 kernels of the FETD-PIC step: positions are kept cell-local as
 // barycentric coordinates (l0, l1; l2 = 1 - l0 - l1), momenta in units of c.
 // Gather, push, walk and deposit run in FP32; particles with gamma > 10 take
-// the FP64 push (Lorentz factor and momentum update), where FP32 loses the
-// 1 - v/c and sigma cancellations.  The field unknowns and the Faraday update
+// the double-float push (Lorentz factor and momentum update), where FP32 loses
+// the 1 - v/c and sigma cancellations.  The field unknowns and the Faraday update
 // stay FP64; the SPAI product of the Ampere update is FP32 (kernels_common.cu).
 //
 // Built with approximate FP32 division and square root (-prec-div=false
@@ -178,22 +178,157 @@ __device__ __forceinline__ T push_c1(T &ux, T &uy, T ex, T ey, T bz)
     return rsq<T, NEWTON>(one + ux * ux + uy * uy);
 }
 
-// FP64 push for gamma > 10 (rare; kept out of line so its registers do not
-// count against the FP32 main path).  Arguments and result by value, so no
-// caller variable needs an address.  Returns (u_x, u_y, v_x, v_y) in units of
-// c and 1/gamma.
-struct PushOut { float ux, uy, vx, vy, ig; };
+// ------------------------------------------------- double-float arithmetic
+// A value held as an unevaluated sum h + l of two floats, |l| <= ulp(h) / 2:
+// 48 significand bits from FP32 additions and fused multiply-adds (Dekker 1971;
+// Knuth's two-sum).  GB300 issues FP32 at 128 lanes per SM and clock and FP64
+// at 2, so the 10-odd FP32 operations of one double-float operation take a
+// sixth of one FP64 instruction's time.  The rounding intrinsics keep the
+// error terms from being contracted.
+struct F2 {
+    float h, l;
+    __device__ __forceinline__ F2() {}
+    __device__ __forceinline__ F2(float a) : h(a), l(0.f) {}
+    __device__ __forceinline__ F2(float a, float b) : h(a), l(b) {}
+};
+__device__ __forceinline__ F2 quick_two_sum(float a, float b)          // |a| >= |b|
+{
+    const float s = __fadd_rn(a, b);
+    return F2(s, __fsub_rn(b, __fsub_rn(s, a)));
+}
+__device__ __forceinline__ F2 two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return F2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t)));
+}
+__device__ __forceinline__ F2 two_prod(float a, float b)
+{
+    const float p = __fmul_rn(a, b);
+    return F2(p, __fmaf_rn(a, b, -p));
+}
+__device__ __forceinline__ F2 operator-(const F2 &a) { return F2(-a.h, -a.l); }
+__device__ __forceinline__ F2 operator+(const F2 &a, const F2 &b)
+{
+    const F2 s = two_sum(a.h, b.h);
+    return quick_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ F2 operator-(const F2 &a, const F2 &b) { return a + (-b); }
+__device__ __forceinline__ F2 operator+(const F2 &a, float b)
+{
+    const F2 s = two_sum(a.h, b);
+    return quick_two_sum(s.h, __fadd_rn(s.l, a.l));
+}
+__device__ __forceinline__ F2 operator*(const F2 &a, const F2 &b)
+{
+    const F2 p = two_prod(a.h, b.h);
+    return quick_two_sum(p.h, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, p.l)));
+}
+__device__ __forceinline__ F2 operator*(const F2 &a, float b)
+{
+    const F2 p = two_prod(a.h, b);
+    return quick_two_sum(p.h, __fmaf_rn(a.l, b, p.l));
+}
+__device__ __forceinline__ F2 sqr(const F2 &a)
+{
+    const F2 p = two_prod(a.h, a.h);
+    return quick_two_sum(p.h, __fmaf_rn(__fadd_rn(a.h, a.h), a.l, p.l));
+}
+// 1/sqrt(x), 1/x: a single-precision seed and one Newton-Raphson step whose
+// residual 1 - x y^2 (1 - x y) is formed without rounding its leading part;
+// relative error about 1e-13, as that of the step in FP64 (the seed's error
+// squared).
+__device__ __forceinline__ F2 rsqrt_f2(const F2 &x)
+{
+    const float y = rsqrtf(x.h);
+    const F2 p = two_prod(x.h, y);                                     // x y
+    const float e = __fmaf_rn(-p.h, y, 1.f) - __fmaf_rn(x.l, y, p.l) * y;
+    return quick_two_sum(y, 0.5f * y * e);
+}
+__device__ __forceinline__ F2 rcp_f2(const F2 &x)
+{
+    const float y = __fdividef(1.f, x.h);
+    return quick_two_sum(y, y * __fmaf_rn(-x.l, y, __fmaf_rn(-x.h, y, 1.f)));
+}
 
+// The push for gamma > 10, where FP32 loses 1 - v/c and the cancellation in
+// sigma: the formulas of push_c1 in double-float (rare in thermal plasmas,
+// every particle of a high-gamma beam; kept out of line so its registers do
+// not count against the FP32 main path).  Arguments and result by value, so no
+// caller variable needs an address.  Returns (u_x, u_y, v_x, v_y) in units of c.
+struct PushOut { float ux, uy, vx, vy; };
+
+// The same in FP64, for what double-float cannot hold: gamma^2 whose square
+// leaves the FP32 range, |beta|^2 close to gamma^2 (sigma cancels), a Boris-tan
+// angle beyond the series.  Inlined into push_f2, where a nested call would
+// cost the particle kernels spills (24 bytes in the Vay kernel at 72 registers);
+// out of line for Boris-tan, whose FP64 tangent costs more than the call.
 template <int PUSHER>
-__device__ __noinline__ PushOut push_fp64(float ux, float uy, float ex, float ey, float bz)
+__device__ __forceinline__ PushOut push_fp64_inl(float ux, float uy, float ex, float ey, float bz)
 {
     double dux = ux, duy = uy;
     const double dig = push_c1<PUSHER, double, true>(dux, duy, (double)ex, (double)ey, (double)bz);
-    PushOut o;
-    o.ux = (float)dux; o.uy = (float)duy;
-    o.vx = (float)(dux * dig); o.vy = (float)(duy * dig);
-    o.ig = (float)dig;
-    return o;
+    return PushOut{(float)dux, (float)duy, (float)(dux * dig), (float)(duy * dig)};
+}
+template <int PUSHER>
+__device__ __noinline__ PushOut push_fp64_call(float ux, float uy, float ex, float ey, float bz)
+{
+    return push_fp64_inl<PUSHER>(ux, uy, ex, ey, bz);
+}
+template <int PUSHER>
+__device__ __forceinline__ PushOut push_fp64(float ux, float uy, float ex, float ey, float bz)
+{
+    if constexpr (PUSHER == FETDPIC_BORIS_TAN) return push_fp64_call<PUSHER>(ux, uy, ex, ey, bz);
+    else return push_fp64_inl<PUSHER>(ux, uy, ex, ey, bz);
+}
+
+template <int PUSHER>
+__device__ __noinline__ PushOut push_f2(float ux, float uy, float ex, float ey, float bz)
+{
+    const F2 bb = two_prod(bz, bz);
+    const F2 umx = two_sum(ux, ex), umy = two_sum(uy, ey);             // u^-
+    const F2 g2 = sqr(umx) + sqr(umy) + 1.f;
+    if (!(g2.h < 1e18f) || !(4.f * bb.h < g2.h)) return push_fp64<PUSHER>(ux, uy, ex, ey, bz);
+    F2 x, y, ig;                                                       // u^{n+1/2}, 1/gamma^{n+1/2}
+    if (PUSHER == FETDPIC_VAY) {
+        const F2 ig0 = rsqrt_f2(two_prod(ux, ux) + two_prod(uy, uy) + 1.f);
+        const F2 upx = umx + ex + ig0 * uy * bz;
+        const F2 upy = umy + ey - ig0 * ux * bz;
+        const F2 sigma = sqr(upx) + sqr(upy) + 1.f - bb;
+        const F2 r2 = sqr(sigma) + F2(4.f * bb.h, 4.f * bb.l);
+        const F2 s2 = sigma + r2 * rsqrt_f2(r2);
+        if (!(sigma.h > 0.f) || !(s2.h < 4e18f)) return push_fp64<PUSHER>(ux, uy, ex, ey, bz);
+        ig = rsqrt_f2(F2(0.5f * s2.h, 0.5f * s2.l));
+        const F2 tz = ig * bz;
+        const F2 s = rcp_f2(sqr(tz) + 1.f);
+        x = s * (upx + upy * tz);
+        y = s * (upy - upx * tz);
+    } else {
+        F2 tz;
+        if (PUSHER == FETDPIC_HC) {
+            const F2 sigma = g2 - bb;
+            const F2 r2 = sqr(sigma) + F2(4.f * bb.h, 4.f * bb.l);
+            const F2 s2 = sigma + r2 * rsqrt_f2(r2);
+            tz = rsqrt_f2(F2(0.5f * s2.h, 0.5f * s2.l)) * bz;
+        } else {
+            tz = rsqrt_f2(g2) * bz;
+            if (PUSHER == FETDPIC_BORIS_TAN) {
+                // tan t = t + t (t^2/3 + 2 t^4/15 + 17 t^6/315 + 62 t^8/2835 + ...): the first
+                // neglected term is below 1e-15 of t for |t| < 0.04
+                if (!(fabsf(tz.h) < 0.04f)) return push_fp64<PUSHER>(ux, uy, ex, ey, bz);
+                const F2 q = sqr(tz);
+                const float r = q.h * q.h * (2.f / 15.f + q.h * (17.f / 315.f + q.h * (62.f / 2835.f)));
+                // 1/3 as a double-float: 1/3 rounded to FP32, and the rest
+                const float third = 1.f / 3.f, rest = (float)(1.0 / 3.0 - (double)third);
+                tz = tz + tz * (q * F2(third, rest) + r);
+            }
+        }
+        const F2 sz = F2(2.f * tz.h, 2.f * tz.l) * rcp_f2(sqr(tz) + 1.f);
+        const F2 uprx = umx + umy * tz, upry = umy - umx * tz;
+        x = umx + upry * sz + ex;
+        y = umy - uprx * sz + ey;
+        ig = rsqrt_f2(sqr(x) + sqr(y) + 1.f);
+    }
+    return PushOut{x.h, y.h, (x * ig).h, (y * ig).h};
 }
 
 // Fixed-point current of one sub-segment, Eq. (I.assign): round(w (l_a^s l_b^f
@@ -470,7 +605,7 @@ struct POne {
     int v[3];                                // fixed-point current if it stays, else 0
 };
 
-// Gather (Sec. II.B), push (Sec. II.C; FP64 when gamma > 10), move in
+// Gather (Sec. II.B), push (Sec. II.C; double-float when gamma > 10), move in
 // barycentrics (Eq. (eq.motion.dis): dl_k = c dt grad l_k . v/c, with
 // dl_2 = -(dl_0 + dl_1) so the barycentrics keep summing to 1), and the
 // current of a particle that stays in its triangle (Eq. (I.assign), written
@@ -486,12 +621,12 @@ __device__ __forceinline__ POne one_particle(float kappa, float wfix, int f, flo
     const float ex = kappa * (l0 * r.r0.x + l1 * r.r0.z + l2 * r.r1.x);
     const float ey = kappa * (l0 * r.r0.y + l1 * r.r0.w + l2 * r.r1.y);
     const float bz = kappa * r.r1.z;
-    float ig, vx, vy;
+    float vx, vy;
     if (1.f + ux * ux + uy * uy > 100.f) {
-        const PushOut q = push_fp64<PUSHER>(ux, uy, ex, ey, bz);
-        ux = q.ux; uy = q.uy; vx = q.vx; vy = q.vy; ig = q.ig;
+        const PushOut q = push_f2<PUSHER>(ux, uy, ex, ey, bz);
+        ux = q.ux; uy = q.uy; vx = q.vx; vy = q.vy;
     } else {
-        ig = push_c1<PUSHER, float>(ux, uy, ex, ey, bz);
+        const float ig = push_c1<PUSHER, float>(ux, uy, ex, ey, bz);
         vx = ux * ig; vy = uy * ig;
     }
     o.bad = live && !isfinite(vx + vy);
