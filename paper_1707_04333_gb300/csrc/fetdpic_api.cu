@@ -77,6 +77,7 @@ struct fetdpic_ctx {
     std::vector<Species> sp;
     Species *sp_dev = nullptr;
     Sp32 *sp32_dev = nullptr;
+    bool soft64 = false;                     // FP64 constants within the integer arithmetic's range
     long long P = 0, nblocks = 0;
     int block = 256;
     int *cell = nullptr, *cell_tmp = nullptr, *id = nullptr, *id_tmp = nullptr;
@@ -650,6 +651,15 @@ static void reset_gauss_reference(fetdpic_ctx *ctx)
     ctx->g0_ready = true;
 }
 
+// Whether the FP64 particle kernel may form products and quotients with `v` in
+// integer arithmetic (fp64_int.h): zero, or a magnitude that leaves chains of
+// them normal.
+static bool soft_constant(double v)
+{
+    const double m = std::fabs(v);
+    return m == 0.0 || (m >= 0x1p-100 && m < 0x1p64);
+}
+
 // Move the staged species to the device: padded species ranges, block ->
 // species table, fixed-point scale of the current per instance.
 static int finalize(fetdpic_ctx *ctx)
@@ -711,6 +721,13 @@ static int finalize(fetdpic_ctx *ctx)
         hist_n += D.nf + 1;                  // the species' triangles, then its padding bin
         off += D.cap;
     }
+    ctx->soft64 = true;
+    for (const Species &D : ctx->sp)
+        ctx->soft64 = ctx->soft64 && soft_constant(D.alpha) && soft_constant(D.ic2) && soft_constant(D.dt) &&
+                      soft_constant(D.wfix);
+    for (const HostMesh &M : ctx->mesh)
+        for (const std::vector<double> *g : {&M.gx, &M.gy, &M.X, &M.Y})
+            ctx->soft64 = ctx->soft64 && std::all_of(g->begin(), g->end(), soft_constant);
     ctx->P = off;
     ctx->nblocks = off / ctx->block;
     if (off >= (1ll << 31))      // particle slots and load indices are 32-bit
@@ -823,14 +840,15 @@ static StepArgs64 args64(fetdpic_ctx *ctx)
 {
     StepArgs64 a{};
     a.geo = ctx->geo64; a.topo = ctx->topo; a.rec = ctx->rec64;
-    a.sp = ctx->sp_dev; a.blk_sp = ctx->blk_sp;
+    a.sp = ctx->sp_dev; a.chunk_sp = ctx->chunk_sp; a.nchunks = ctx->P / 32;
+    a.soft = ctx->soft64; a.ext_on = ctx->ext_on;
     a.x = (double *)ctx->f[0]; a.y = (double *)ctx->f[1]; a.ux = (double *)ctx->f[2]; a.uy = (double *)ctx->f[3];
     a.cell = ctx->cell;
     a.ifix = ctx->ifix; a.status = ctx->status;
     a.max_cross = ctx->p.max_crossings;
     a.rec_cap = ctx->p.record_walk; a.rec_cnt = ctx->rec_cnt; a.wrec = ctx->rec; a.id = ctx->id;
     a.edge_off = ctx->edge_off_dev;
-    a.nblocks = ctx->nblocks; a.block = ctx->block;
+    a.block = ctx->block;
     a.tshift = ctx->tshift; a.period = ctx->period;
     a.extw = ctx->extw; a.ext_amp = ctx->ext_amp;
     return a;

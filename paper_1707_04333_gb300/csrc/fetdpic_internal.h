@@ -187,7 +187,7 @@ __device__ __forceinline__ void pdl_begin()
 
 struct StepArgs64 {
     const Geo64 *geo; const Topo *topo; const Rec64 *rec;
-    const Species *sp; const short *blk_sp;
+    const Species *sp; const short *chunk_sp;   // species of each 32-particle chunk
     double *x, *y, *ux, *uy; int *cell;
     unsigned long long *ifix;               // [E] fixed-point current (two's complement)
     unsigned *status;
@@ -197,7 +197,9 @@ struct StepArgs64 {
                                             // after the step does not move it
     const int *id;                          // load index of each particle slot
     const int *edge_off;                    // per instance, for instance-local record ids
-    long long nblocks; int block;
+    long long nchunks; int block;
+    bool soft;                              // geometry and species constants suit the integer arithmetic
+    bool ext_on;                            // some applied field or profile is set
     const signed char *tshift;              // [F][3] periodic shift codes; NULL = no periodic walls
     const double2 *period;                  // per instance (tx, ty)
     const double2 *extw;                    // [F] weights (E, B) of the applied fields; NULL = 1

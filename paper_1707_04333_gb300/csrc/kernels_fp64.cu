@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "fetdpic_internal.h"
+#include "fp64_int.h"
 
 namespace fetdpic {
 
@@ -48,6 +49,48 @@ void launch_faraday64(cudaStream_t st, int F, const Geo64 *geo, const Topo *topo
     k_faraday64<<<(F + 255) / 256, 256, 0, st>>>(F, geo, topo, e, b, rec);
 }
 
+// ------------------------------------------------------------ arithmetic
+// The particle kernel's arithmetic comes in two forms with the same bits: the
+// hardware's FP64 instructions, and multiplication, division, square root and
+// the conversion to integers in 32-bit integer instructions (fp64_int.h), with
+// additions and a few products left on the FP64 pipe (about as many as balance
+// the two).  GB300's FP64 pipe passes 2 lanes per SM and clock and bounded the
+// hardware form (83 % busy, the schedulers 8 %).
+// The integer form takes operands whose products and quotients stay normal;
+// a particle with others (checked as they are loaded) takes the hardware form.
+struct Hard {
+    static constexpr bool SOFT = false;
+    static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
+    static __device__ __forceinline__ double div(double a, double b) { return a / b; }
+    static __device__ __forceinline__ double root(double a) { return sqrt(a); }
+    static __device__ __forceinline__ double twice(double a) { return 2.0 * a; }
+    static __device__ __forceinline__ double half(double a) { return 0.5 * a; }
+    static __device__ __forceinline__ double four(double a) { return 4.0 * a; }
+    static __device__ __forceinline__ long long round(double a) { return __double2ll_rn(a); }
+    static __device__ __forceinline__ bool neg(double a) { return a < 0.0; }
+};
+// (Out of line, and the loops over the three nodes or edges left rolled: the
+// straight-line form of a push is about 3,500 instructions, and its warps then
+// wait for instructions more than for anything else.)
+__device__ __noinline__ double div_call(double a, double b) { return div_i(a, b); }
+__device__ __noinline__ double root_call(double a) { return sqrt_i(a); }
+struct Soft {
+    static constexpr bool SOFT = true;
+    static __device__ __forceinline__ double mul(double a, double b) { return mul_i(a, b); }
+    static __device__ __forceinline__ double div(double a, double b) { return div_call(a, b); }
+    static __device__ __forceinline__ double root(double a) { return root_call(a); }
+    static __device__ __forceinline__ double twice(double a) { return scale_i<1>(a); }
+    static __device__ __forceinline__ double half(double a) { return scale_i<-1>(a); }
+    static __device__ __forceinline__ double four(double a) { return scale_i<2>(a); }
+    // an addition rounds |a| < 2^51 to an integer in its low bits
+    static __device__ __forceinline__ long long round(double a)
+    {
+        if ((f64_hi(a) & 0x7fffffffu) >= ((1023u + 51u) << 20)) return rint_i(a);
+        return __double_as_longlong(a + 0x1.8p52) - __double_as_longlong(0x1.8p52);
+    }
+    static __device__ __forceinline__ bool neg(double a) { return is_neg(a); }
+};
+
 // ------------------------------------------------------------------ push
 // 2-D TE specialisation (u_z = 0, E_z = 0, B along z) of the 3-vector
 // formulas of Sec. II.C; with u_z = 0 every dropped term is an exact zero,
@@ -55,59 +98,70 @@ void launch_faraday64(cudaStream_t st, int F, const Geo64 *geo, const Topo *topo
 
 struct Push { double ux, uy, g; };
 
+template <class A>
 __device__ __forceinline__ double gam2(double ux, double uy, double ic2)
 {
-    return sqrt(1.0 + (ux * ux + uy * uy) * ic2);
+    return A::root(1.0 + A::mul(A::mul(ux, ux) + A::mul(uy, uy), ic2));
 }
 
-template <int PUSHER>
+// `ok` (integer form): cleared when u' or u^- leaves the range the rest is safe for.
+template <class A, int PUSHER>
 __device__ __forceinline__ Push push64(double ux, double uy, double Ex, double Ey, double Bz,
-                                       double alpha, double c, double ic2)
+                                       double alpha, double ic2, bool &ok)
 {
-    const double epsx = alpha * Ex, epsy = alpha * Ey;
-    const double bz = alpha * Bz;
-    const double bb = bz * bz;
+    const double epsx = A::mul(alpha, Ex), epsy = A::mul(alpha, Ey);
+    const double bz = A::mul(alpha, Bz);
+    const double bb = A::mul(bz, bz);
     Push out;
     if (PUSHER == FETDPIC_VAY) {
         // Sec. II.C(b): u^n = u^{n-1/2} + eps + v^{n-1/2} x beta; u' = u^n + eps;
         // gamma^{n+1/2} from the quartic; u^{n+1/2} = s (u' + (u'.t) t + u' x t), s = 1/(1+t^2)
-        const double g0 = gam2(ux, uy, ic2);
-        const double vx = ux / g0, vy = uy / g0;
-        const double unx = (ux + epsx) + vy * bz;
-        const double uny = (uy + epsy) - vx * bz;
+        const double g0 = gam2<A>(ux, uy, ic2);
+        const double vx = A::div(ux, g0), vy = A::div(uy, g0);
+        const double unx = (ux + epsx) + A::mul(vy, bz);
+        const double uny = (uy + epsy) - A::mul(vx, bz);
         const double upx = unx + epsx, upy = uny + epsy;
-        const double gp = gam2(upx, upy, ic2);
-        const double sigma = gp * gp - bb;
-        const double gn = sqrt(0.5 * (sigma + sqrt(sigma * sigma + 4.0 * bb)));
-        const double tz = bz / gn;
-        const double s = 1.0 / (1.0 + tz * tz);
-        out.ux = s * (upx + upy * tz);
-        out.uy = s * (upy - upx * tz);
+        if (A::SOFT) ok = ok && f64_within<120, 64>(upx) && f64_within<120, 64>(upy);
+        const double gp = gam2<A>(upx, upy, ic2);
+        const double sigma = A::mul(gp, gp) - bb;
+        const double gn = A::root(A::half(sigma + A::root(A::mul(sigma, sigma) + A::four(bb))));
+        const double tz = A::div(bz, gn);
+        const double s = A::div(1.0, 1.0 + A::mul(tz, tz));
+        out.ux = A::mul(s, upx + A::mul(upy, tz));
+        out.uy = A::mul(s, upy - A::mul(upx, tz));
         out.g = gn;
         return out;
     }
     // Boris family, Eqs. (Boris.u1-u4)
     const double umx = ux + epsx, umy = uy + epsy;
-    const double gbar = gam2(umx, umy, ic2);                 // Eq. (gamma.middle)
+    if (A::SOFT) ok = ok && f64_within<120, 64>(umx) && f64_within<120, 64>(umy);
+    const double gbar = gam2<A>(umx, umy, ic2);              // Eq. (gamma.middle)
     double tz;
     if (PUSHER == FETDPIC_HC) {
         // Sec. II.C(c): gamma_H from sigma = gamma_B^2 - |beta|^2 (u^- . beta = 0 in 2-D TE)
-        const double sigma = gbar * gbar - bb;
-        const double gh = sqrt(0.5 * (sigma + sqrt(sigma * sigma + 4.0 * bb)));
-        tz = bz / gh;
+        const double sigma = A::mul(gbar, gbar) - bb;
+        const double gh = A::root(A::half(sigma + A::root(A::mul(sigma, sigma) + A::four(bb))));
+        tz = A::div(bz, gh);
     } else if (PUSHER == FETDPIC_BORIS_TAN) {
-        const double nb = sqrt(bb);
-        tz = (nb == 0.0) ? 0.0 : (bz / nb) * tan(nb / gbar);
+        // (sqrt(bz^2) and bz / |bz| are exact where bz^2 does not underflow)
+        const double nb = A::SOFT ? fabs(bz) : sqrt(bb);
+        if (A::SOFT) {
+            const double t = tan(A::div(nb, gbar));
+            tz = is_neg(bz) ? -t : t;
+        } else {
+            tz = (nb == 0.0) ? 0.0 : (bz / nb) * tan(nb / gbar);
+        }
     } else {
-        tz = bz / gbar;
+        tz = A::div(bz, gbar);
     }
-    const double den = 1.0 + tz * tz;
-    const double sz = (2.0 * tz) / den;
-    const double uprx = umx + umy * tz, upry = umy - umx * tz;   // u' = u^- + u^- x t
-    const double upx = umx + upry * sz, upy = umy - uprx * sz;   // u^+ = u^- + u' x s
+    const double den = 1.0 + A::mul(tz, tz);
+    const double sz = A::div(A::twice(tz), den);
+    const double uprx = umx + A::mul(umy, tz), upry = umy - A::mul(umx, tz);   // u' = u^- + u^- x t
+    const double upx = umx + A::mul(upry, sz), upy = umy - A::mul(uprx, sz);   // u^+ = u^- + u' x s
     out.ux = upx + epsx;
     out.uy = upy + epsy;
-    out.g = gam2(out.ux, out.uy, ic2);
+    if (A::SOFT) ok = ok && f64_within<120, 64>(out.ux) && f64_within<120, 64>(out.uy);
+    out.g = gam2<A>(out.ux, out.uy, ic2);
     return out;
 }
 
@@ -121,242 +175,213 @@ __device__ __forceinline__ void red_add_u64(unsigned long long *p, long long v)
 // Fixed-point current of one sub-segment, Eq. (I.assign): for local edge m
 // with (a, b) = (m+1, m+2), (Q/dt)(l_a^s l_b^f - l_a^f l_b^s), scaled by
 // 2^shift/(Q_ref/dt) and rounded to the nearest integer.
+template <class A>
 __device__ __forceinline__ void seg_current(const double *ls, const double *lf, double w, long long *v)
 {
-#pragma unroll
+    // l(m+1), l(m+2) of round m; the values rotate through registers
+    double sa = ls[1], sb = ls[2], sc = ls[0], fa = lf[1], fb = lf[2], fc = lf[0];
+#pragma unroll 1
     for (int m = 0; m < 3; ++m) {
-        const int a = (m + 1) % 3, b = (m + 2) % 3;
-        const double d = ls[a] * lf[b] - lf[a] * ls[b];
-        v[m] = __double2ll_rn(d * w);
-    }
-}
-
-__device__ __forceinline__ void add_seg(unsigned long long *ifix, const Topo &t, const long long *v)
-{
-#pragma unroll
-    for (int m = 0; m < 3; ++m) {
-        const long long s = (t.ew[m] & 1) ? -v[m] : v[m];
-        red_add_u64(ifix + (t.ew[m] >> 1), s);
+        const double d = A::mul(sa, fb) - A::mul(fa, sb);
+        const long long r = A::round(d * w);
+        v[0] = v[1]; v[1] = v[2]; v[2] = r;
+        const double s = sa, f = fa;
+        sa = sb; sb = sc; sc = s;
+        fa = fb; fb = fc; fc = f;
     }
 }
 
 // --------------------------------------------------------- particle kernel
-// One thread per particle.  Blocks never straddle species (species storage
-// ranges are padded to 1024).  The first sub-segment of every particle (in
-// its starting triangle) is reduced across the warp over runs of equal
-// triangle (particles are sorted by triangle), so one lane per run issues the
-// three 64-bit integer additions; the rare further sub-segments add directly.
-// Integer addition is associative, so the result does not depend on the
-// order of particles or atomics: deposits are deterministic.
-template <int PUSHER>
-__global__ void __launch_bounds__(256) k_particles64(StepArgs64 a)
+
+// 32 bytes in one 256-bit load (read-only data).
+__device__ __forceinline__ void ld_4d(const double *p, double &a, double &b, double &c, double &d)
 {
-    __shared__ Species S;
-    const long long blk = blockIdx.x;
-    if (threadIdx.x == 0) S = a.sp[a.blk_sp[blk]];
-    __syncthreads();
-    const long long p = blk * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    int f = a.cell[p];
-    const bool live = f >= 0;
+    asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p));
+}
+struct Tri64 { double gx[3], gy[3], X[3], Y[3]; };
+__device__ __forceinline__ Tri64 load_tri(const Geo64 *g)
+{
+    const double *d = reinterpret_cast<const double *>(g);
+    Tri64 t;
+    ld_4d(d, t.gx[0], t.gx[1], t.gx[2], t.gy[0]);
+    ld_4d(d + 4, t.gy[1], t.gy[2], t.X[0], t.X[1]);
+    ld_4d(d + 8, t.X[2], t.Y[0], t.Y[1], t.Y[2]);
+    return t;
+}
+template <class A>
+__device__ __forceinline__ void lambdas(const Tri64 &t, double x, double y, double *l)
+{
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        const int an = (m + 1) % 3;
+        l[m] = A::mul(t.gx[m], x - t.X[an]) + A::mul(t.gy[m], y - t.Y[an]);
+    }
+}
 
-    long long v0[3] = {0, 0, 0};
-    Topo t0;
-    int key = -1;
-    bool walking = false;
-    // walk state (carried into the divergent continuation)
-    double xs = 0, ys = 0, xf = 0, yf = 0, ux = 0, uy = 0, tin = 0.0;
-    double lin[3] = {0, 0, 0};
-    int min = -1, ncross = 0;
-    const double *gxp = nullptr, *gyp = nullptr;
-    Topo tc;
-    // walk record slot: species storage offset + load index (unmoved by a later sort)
-    const long long rp = (a.rec_cap > 0 && live) ? S.off + a.id[p] : 0;
+// One particle's gather, push, end point and, if it stays in its triangle, its
+// current.  ok: false when the integer form met an operand it does not take.
+struct One64 {
+    double xf, yf, ux, uy;
+    long long v[3];
+    bool stays, ok;
+};
 
-    if (live) {
-        const Geo64 &G = a.geo[f];
-        tc = a.topo[f];
-        const Rec64 R = a.rec[f];
-        xs = a.x[p]; ys = a.y[p];
-        ux = a.ux[p]; uy = a.uy[p];
-        double gx[3], gy[3], X[3], Y[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) { gx[k] = G.gx[k]; gy[k] = G.gy[k]; X[k] = G.X[k]; Y[k] = G.Y[k]; }
-        double lam[3];
-#pragma unroll
+template <class A, int PUSHER>
+__device__ __forceinline__ One64 one_particle64(const StepArgs64 &a, const Species *S, int f, double xs, double ys,
+                                                double ux, double uy)
+{
+    One64 o;
+    const Tri64 t = load_tri(a.geo + f);
+    Rec64 R;
+    ld_4d(a.rec[f].se, R.se[0], R.se[1], R.se[2], R.bz);
+    o.ok = true;
+    if (A::SOFT) {
+        // E may be a far wave's tail (it enters linearly), B and the momentum are squared
+        o.ok = f64_within<120, 64>(xs) && f64_within<120, 64>(ys) && f64_within<120, 64>(ux) &&
+               f64_within<120, 64>(uy) && f64_within<400, 64>(R.se[0]) && f64_within<400, 64>(R.se[1]) &&
+               f64_within<400, 64>(R.se[2]);
+    }
+    double lam[3];
+    lambdas<A>(t, xs, ys, lam);
+    // gather E^n (Sec. II.B): sum_m s_m e_m (l_a grad l_b - l_b grad l_a)
+    double Ex = 0.0, Ey = 0.0;
+    {
+        double la = lam[1], lb = lam[2], lc = lam[0], xa = t.gx[1], xb = t.gx[2], xc = t.gx[0], ya = t.gy[1],
+               yb = t.gy[2], yc = t.gy[0], ea = R.se[0], eb = R.se[1];
+        const double ec = R.se[2];
+#pragma unroll 1
         for (int m = 0; m < 3; ++m) {
-            const int an = (m + 1) % 3;
-            lam[m] = gx[m] * (xs - X[an]) + gy[m] * (ys - Y[an]);
+            const double wx = A::mul(la, xb) - A::mul(lb, xa);
+            const double wy = A::mul(la, yb) - A::mul(lb, ya);
+            Ex = Ex + ea * wx;                                         // on the FP64 pipe in both forms
+            Ey = Ey + ea * wy;
+            const double l = la, x = xa, y = ya;
+            la = lb; lb = lc; lc = l;
+            xa = xb; xb = xc; xc = x;
+            ya = yb; yb = yc; yc = y;
+            ea = eb; eb = ec;
         }
-        // gather E^n (Sec. II.B): sum_m s_m e_m (l_a grad l_b - l_b grad l_a)
-        double Ex = 0.0, Ey = 0.0;
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            const int an = (m + 1) % 3, bn = (m + 2) % 3;
-            const double wx = lam[an] * gx[bn] - lam[bn] * gx[an];
-            const double wy = lam[an] * gy[bn] - lam[bn] * gy[an];
-            Ex = Ex + R.se[m] * wx;
-            Ey = Ey + R.se[m] * wy;
-        }
+    }
+    double Bz = R.bz;
+    if (a.ext_on) {
         // applied fields: (amplitude x E weight) E_ext, B weight x B_ext in this triangle
         double we = 1.0, wb = 1.0;
         if (a.extw) { const double2 wv = a.extw[f]; we = wv.x; wb = wv.y; }
-        const double sa = a.ext_amp[S.inst] * we;
-        Ex = Ex + sa * S.ext_ex;
-        Ey = Ey + sa * S.ext_ey;
-        const double Bz = R.bz + wb * S.ext_bz;
-        const Push u = push64<PUSHER>(ux, uy, Ex, Ey, Bz, S.alpha, S.c, S.ic2);
-        ux = u.ux; uy = u.uy;
-        if (!isfinite(u.g) || !isfinite(ux) || !isfinite(uy)) atomicOr(a.status, (unsigned)ST_NONFINITE);
-        const double ig = 1.0 / u.g;
-        xf = xs + (ux * ig) * S.dt;                         // Eq. (eq.motion.dis)
-        yf = ys + (uy * ig) * S.dt;
-        lin[0] = lam[0]; lin[1] = lam[1]; lin[2] = lam[2];
+        const double sa = a.ext_amp[S->inst] * we;
+        Ex = Ex + sa * S->ext_ex;
+        Ey = Ey + sa * S->ext_ey;
+        Bz = R.bz + wb * S->ext_bz;
+        if (A::SOFT) o.ok = o.ok && f64_within<700, 300>(Ex) && f64_within<700, 300>(Ey);
+    }
+    if (A::SOFT) o.ok = o.ok && f64_within<120, 64>(Bz);
+    const Push u = push64<A, PUSHER>(ux, uy, Ex, Ey, Bz, S->alpha, S->ic2, o.ok);
+    o.ux = u.ux; o.uy = u.uy;
+    if (!A::SOFT) {
+        if (!isfinite(u.g) || !isfinite(u.ux) || !isfinite(u.uy)) atomicOr(a.status, (unsigned)ST_NONFINITE);
+    }
+    const double ig = A::div(1.0, u.g);
+    const double dt = S->dt;
+    o.xf = xs + A::mul(A::mul(u.ux, ig), dt);                   // Eq. (eq.motion.dis)
+    o.yf = ys + A::mul(A::mul(u.uy, ig), dt);
+    // the geometry is read again (L1) rather than kept through the push: 24 registers
+    double lf[3];
+    lambdas<A>(load_tri(a.geo + f), o.xf, o.yf, lf);
+    o.stays = !(A::neg(lf[0]) || A::neg(lf[1]) || A::neg(lf[2]));
+    seg_current<A>(lam, lf, S->wfix, o.v);
+    return o;
+}
 
-        // first sub-segment, in the starting triangle
+// The hardware form for a particle the integer form does not take (out of line: rare).
+template <int PUSHER>
+__device__ __noinline__ One64 one_particle64_hard(const StepArgs64 &a, const Species *S, int f, double xs, double ys,
+                                                  double ux, double uy)
+{
+    return one_particle64<Hard, PUSHER>(a, S, f, xs, ys, ux, uy);
+}
+
+// A particle whose path leaves its starting triangle, queued per warp.
+struct __align__(16) Walk64 {
+    double xs, ys, xf, yf, ux, uy;
+    unsigned p;                              // particle slot
+    int f;                                   // starting triangle
+    int soft, pad;                           // the integer form took its push
+};
+static_assert(sizeof(Walk64) == 64, "Walk64 layout");
+constexpr int RING64 = 64;                   // 31 pending + 32 new fit
+
+// Walk of a queued particle through the triangles it crosses: exit test,
+// deposit of each sub-segment, hand-off to the neighbour or specular
+// reflection at a PEC wall, and the final particle state.  The integer current
+// of a crossed edge is carried to the next sub-segment, which ends on the same
+// edge: one atomic, not two.
+template <class A>
+__device__ __forceinline__ void walk64(const StepArgs64 &a, const Walk64 &it)
+{
+    const unsigned p = it.p;
+    const Species *S = a.sp + a.chunk_sp[p >> 5];
+    // walk record slot: species storage offset + load index (unmoved by a later sort)
+    const long long rp = a.rec_cap > 0 ? S->off + a.id[p] : 0;
+    const int inst = S->inst;
+    const double wfix = S->wfix;
+    double xs = it.xs, ys = it.ys, xf = it.xf, yf = it.yf, ux = it.ux, uy = it.uy, tin = 0.0;
+    double lin[3];
+    int f = it.f, min = -1, ncross = 0;
+    bool first = true, reflected = false;
+    long long carry = 0;                     // current on the entry edge, not yet deposited
+    for (;;) {
+        const Tri64 t = load_tri(a.geo + f);
+        const Topo *tp = a.topo + f;
+        const int ew[3] = {__ldg(&tp->ew[0]), __ldg(&tp->ew[1]), __ldg(&tp->ew[2])};
         double ls[3], lf[3];
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            const int an = (m + 1) % 3;
-            ls[m] = gx[m] * (xs - X[an]) + gy[m] * (ys - Y[an]);
-            lf[m] = gx[m] * (xf - X[an]) + gy[m] * (yf - Y[an]);
-        }
+        lambdas<A>(t, xs, ys, ls);
+        lambdas<A>(t, xf, yf, lf);
+        if (first) { lin[0] = ls[0]; lin[1] = ls[1]; lin[2] = ls[2]; first = false; }
+        // candidate exits in ascending order; a warp runs as many rounds as its worst lane has
+        unsigned cand = (A::neg(lf[0]) ? 1u : 0u) | (A::neg(lf[1]) ? 2u : 0u) | (A::neg(lf[2]) ? 4u : 0u);
+        if (min >= 0) cand &= ~(1u << min);
         int best = -1;
         double tb = 0.0;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            if (lf[k] < 0.0) {
-                const double den = ls[k] - lf[k];
-                double t = den > 0.0 ? ls[k] / den : tin;
-                if (t < tin) t = tin;
-                if (best < 0 || t < tb) { best = k; tb = t; }
-            }
-        }
-        t0 = tc;
-        key = f;
-        if (best < 0) {
-            seg_current(lin, lf, S.wfix, v0);
-        } else {
-            double lout[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) lout[k] = ls[k] + tb * (lf[k] - ls[k]);
-            lout[best] = 0.0;
-            seg_current(lin, lout, S.wfix, v0);
-            walking = true;
-            // hand-off (shared with the divergent loop below)
-            const int eg = tc.ew[best] >> 1;
-            if (ncross >= a.max_cross) {
-                xf = xs + tb * (xf - xs); yf = ys + tb * (yf - ys);
-                atomicOr(a.status, (unsigned)ST_WALK);
-                walking = false;
-            } else {
-                const int nbw = tc.nb[best];
-                if (a.rec_cap > ncross) a.wrec[rp * a.rec_cap + ncross] = nbw < 0 ? -(eg - a.edge_off[S.inst] + 1) : eg - a.edge_off[S.inst];
-                ++ncross;
-                if (nbw < 0) {
-                    const double xw = xs + tb * (xf - xs), yw = ys + tb * (yf - ys);
-                    const double gxb = gx[best], gyb = gy[best];
-                    const double gg = gxb * gxb + gyb * gyb;
-                    const double pr = ((xf - xw) * gxb + (yf - yw) * gyb) / gg;
-                    xf = xf - 2.0 * pr * gxb;
-                    yf = yf - 2.0 * pr * gyb;
-                    const double pu = (ux * gxb + uy * gyb) / gg;
-                    ux = ux - 2.0 * pu * gxb;
-                    uy = uy - 2.0 * pu * gyb;
-                    xs = xw; ys = yw;
-                    tin = 0.0;
-                    min = best;
-                    lin[0] = lout[0]; lin[1] = lout[1]; lin[2] = lout[2];
-                } else {
-                    const int g2 = nbw >> 2, m2 = nbw & 3;
-                    double l2[3];
-                    l2[m2] = 0.0;
-                    l2[(m2 + 1) % 3] = lout[(best + 2) % 3];
-                    l2[(m2 + 2) % 3] = lout[(best + 1) % 3];
-                    lin[0] = l2[0]; lin[1] = l2[1]; lin[2] = l2[2];
-                    if (a.tshift) {
-                        // periodic wall: the rest of the segment continues from the other copy
-                        const int sc = a.tshift[3 * f + best];
-                        if (sc != 0) {
-                            const double2 T = a.period[tc.inst];
-                            xs = xs + sc * T.x; ys = ys + sc * T.y;
-                            xf = xf + sc * T.x; yf = yf + sc * T.y;
-                        }
-                    }
-                    f = g2;
-                    min = m2;
-                    tin = tb;
-                    tc = a.topo[f];
-                }
-            }
-        }
-    }
-
-    // warp segmented reduction of the first sub-segment over runs of equal triangle
-    {
-        const unsigned full = 0xffffffffu;
-        const int kn = __shfl_down_sync(full, key, 1);
-        const bool tail = (lane == 31) || (kn != key);
-        const unsigned tails = __ballot_sync(full, tail);
-        const int seg_end = lane + __ffs(tails >> lane) - 1;
-        const int kp = __shfl_up_sync(full, key, 1);
-        const bool head = (lane == 0) || (kp != key);
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                const long long o = __shfl_down_sync(full, v0[m], off);
-                if (lane + off <= seg_end) v0[m] += o;
-            }
-        }
-        if (head && key >= 0) add_seg(a.ifix, t0, v0);
-    }
-
-    // divergent continuation of the walk (rare: particles that left their triangle)
-    while (walking) {
-        const Geo64 &G = a.geo[f];
-        gxp = G.gx; gyp = G.gy;
-        double ls[3], lf[3];
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            const int an = (m + 1) % 3;
-            ls[m] = gxp[m] * (xs - G.X[an]) + gyp[m] * (ys - G.Y[an]);
-            lf[m] = gxp[m] * (xf - G.X[an]) + gyp[m] * (yf - G.Y[an]);
-        }
-        int best = -1;
-        double tb = 0.0;
-        for (int k = 0; k < 3; ++k) {
-            if (k == min) continue;
-            if (lf[k] < 0.0) {
-                const double den = ls[k] - lf[k];
-                double t = den > 0.0 ? ls[k] / den : tin;
-                if (t < tin) t = tin;
-                if (best < 0 || t < tb) { best = k; tb = t; }
-            }
-        }
-        long long v[3];
-        if (best < 0) {
-            seg_current(lin, lf, S.wfix, v);
-            add_seg(a.ifix, tc, v);
-            break;
+        while (cand) {
+            const int k = __ffs(cand) - 1;
+            cand &= cand - 1u;
+            const double s = k == 0 ? ls[0] : k == 1 ? ls[1] : ls[2];
+            const double den = s - (k == 0 ? lf[0] : k == 1 ? lf[1] : lf[2]);
+            double tk = den > 0.0 ? A::div(s, den) : tin;
+            if (tk < tin) tk = tin;
+            if (best < 0 || tk < tb) { best = k; tb = tk; }
         }
         double lout[3];
-        for (int k = 0; k < 3; ++k) lout[k] = ls[k] + tb * (lf[k] - ls[k]);
-        lout[best] = 0.0;
-        seg_current(lin, lout, S.wfix, v);
-        add_seg(a.ifix, tc, v);
-        const int eg = tc.ew[best] >> 1;
+        if (best < 0) {
+            lout[0] = lf[0]; lout[1] = lf[1]; lout[2] = lf[2];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) lout[k] = k == best ? 0.0 : ls[k] + A::mul(tb, lf[k] - ls[k]);
+        }
+        long long v[3];
+        seg_current<A>(lin, lout, wfix, v);
+        const long long cin = carry;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            long long s = (ew[m] & 1) ? -v[m] : v[m];
+            if (m == min) s += cin;
+            if (m == best) carry = s;
+            else red_add_u64(a.ifix + (ew[m] >> 1), s);
+        }
+        if (best < 0) break;
+        const int eg = (best == 0 ? ew[0] : best == 1 ? ew[1] : ew[2]) >> 1;
         if (ncross >= a.max_cross) {
-            xf = xs + tb * (xf - xs); yf = ys + tb * (yf - ys);
+            red_add_u64(a.ifix + eg, carry);
+            xf = xs + A::mul(tb, xf - xs); yf = ys + A::mul(tb, yf - ys);
             atomicOr(a.status, (unsigned)ST_WALK);
             break;
         }
-        const int nbw = tc.nb[best];
-        if (a.rec_cap > ncross) a.wrec[rp * a.rec_cap + ncross] = nbw < 0 ? -(eg - a.edge_off[S.inst] + 1) : eg - a.edge_off[S.inst];
+        const int nbw = __ldg(&tp->nb[best]);
+        if (a.rec_cap > ncross) a.wrec[rp * a.rec_cap + ncross] = nbw < 0 ? -(eg - a.edge_off[inst] + 1) : eg - a.edge_off[inst];
         ++ncross;
         if (nbw < 0) {
-            const double xw = xs + tb * (xf - xs), yw = ys + tb * (yf - ys);
-            const double gxb = gxp[best], gyb = gyp[best];
+            const double xw = xs + A::mul(tb, xf - xs), yw = ys + A::mul(tb, yf - ys);
+            const double gxb = best == 0 ? t.gx[0] : best == 1 ? t.gx[1] : t.gx[2];
+            const double gyb = best == 0 ? t.gy[0] : best == 1 ? t.gy[1] : t.gy[2];
             const double gg = gxb * gxb + gyb * gyb;
             const double pr = ((xf - xw) * gxb + (yf - yw) * gyb) / gg;
             xf = xf - 2.0 * pr * gxb;
@@ -368,45 +393,162 @@ __global__ void __launch_bounds__(256) k_particles64(StepArgs64 a)
             tin = 0.0;
             min = best;
             lin[0] = lout[0]; lin[1] = lout[1]; lin[2] = lout[2];
+            reflected = true;
         } else {
-            const int g2 = nbw >> 2, m2 = nbw & 3;
-            double l2[3];
-            l2[m2] = 0.0;
-            l2[(m2 + 1) % 3] = lout[(best + 2) % 3];
-            l2[(m2 + 2) % 3] = lout[(best + 1) % 3];
-            lin[0] = l2[0]; lin[1] = l2[1]; lin[2] = l2[2];
+            // hand-off: the neighbour's node m2+1 is our node best+2, its m2+2 our best+1
+            const int m2 = nbw & 3;
+            const double la = best == 0 ? lout[2] : best == 1 ? lout[0] : lout[1];
+            const double lb = best == 0 ? lout[1] : best == 1 ? lout[2] : lout[0];
+            lin[0] = m2 == 0 ? 0.0 : (m2 == 2 ? la : lb);
+            lin[1] = m2 == 1 ? 0.0 : (m2 == 0 ? la : lb);
+            lin[2] = m2 == 2 ? 0.0 : (m2 == 1 ? la : lb);
             if (a.tshift) {
+                // periodic wall: the rest of the segment continues from the other copy
                 const int sc = a.tshift[3 * f + best];
                 if (sc != 0) {
-                    const double2 T = a.period[tc.inst];
+                    const double2 T = a.period[inst];
                     xs = xs + sc * T.x; ys = ys + sc * T.y;
                     xf = xf + sc * T.x; yf = yf + sc * T.y;
                 }
             }
-            f = g2;
+            f = nbw >> 2;
             min = m2;
             tin = tb;
-            tc = a.topo[f];
         }
     }
+    a.x[p] = xf; a.y[p] = yf;
+    if (reflected) { a.ux[p] = ux; a.uy[p] = uy; }
+    a.cell[p] = f;
+    if (a.rec_cap > 0) a.rec_cnt[rp] = ncross;
+}
 
-    if (live) {
-        a.x[p] = xf; a.y[p] = yf;
-        a.ux[p] = ux; a.uy[p] = uy;
-        a.cell[p] = f;
-        if (a.rec_cap > 0) a.rec_cnt[rp] = ncross;
+__device__ __noinline__ void walk64_hard(const StepArgs64 &a, const Walk64 *it) { walk64<Hard>(a, *it); }
+__device__ __noinline__ void walk64_soft(const StepArgs64 &a, const Walk64 *it) { walk64<Soft>(a, *it); }
+
+__device__ __forceinline__ void walk64_any(const StepArgs64 &a, const Walk64 *it)
+{
+    if (it->soft) walk64_soft(a, it);
+    else walk64_hard(a, it);
+}
+
+// Persistent warps, each over a contiguous range of 32-particle chunks (a chunk
+// never straddles species), one particle per lane.  The current of the particles that
+// stay in their triangle is summed over runs of equal triangle (particles are
+// sorted by triangle) by shuffles, one lane per run issuing the three 64-bit
+// integer additions; walkers go to the warp's ring in shared memory and are
+// walked 32 at a time (a divergent walk per chunk ran the FP64 instructions of
+// every chunk's two or three walkers on a whole warp's time).  Integer
+// addition is associative, so the result does not depend on the order of
+// particles or atomics: deposits are deterministic.
+//
+// Bound by the FP64 pipe (59 % busy with the additions and nine products) and
+// the integer pipe (51 %) together.  128 registers and 16 warps per SM: at 80
+// registers (24 warps) the spills cost what the warps bring.  2.05 M particles,
+// Higuera-Cary: 1052 -> 390 us a launch; 327,680, Vay: 203 -> 76 us.
+template <int PUSHER>
+__global__ void __launch_bounds__(256, 2) k_particles64(StepArgs64 a)
+{
+    extern __shared__ Walk64 rings[];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    Walk64 *q = rings + warp * RING64;
+    unsigned qhead = 0, qtail = 0;                        // warp-uniform ring positions
+    const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
+    const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
+    long long c = wid * a.nchunks / nwarps;
+    const long long cend = (wid + 1) * a.nchunks / nwarps;
+    for (; c < cend; ++c) {
+        const long long p = c * 32 + lane;
+        const int f = a.cell[p];
+        const double xs = a.x[p], ys = a.y[p], ux = a.ux[p], uy = a.uy[p];
+        const Species *S = a.sp + a.chunk_sp[c];
+        const bool live = f >= 0;
+        One64 o;
+        o.ok = false;
+        if (a.soft && live) o = one_particle64<Soft, PUSHER>(a, S, f, xs, ys, ux, uy);
+        const bool soft = o.ok;
+        if (live && !soft) o = one_particle64_hard<PUSHER>(a, S, f, xs, ys, ux, uy);
+        const bool stays = live && o.stays, walks = live && !o.stays;
+        {
+            const unsigned wm = __ballot_sync(full, walks);
+            if (walks) {
+                Walk64 &w = q[(qtail + __popc(wm & ((1u << lane) - 1u))) & (RING64 - 1)];
+                w.xs = xs; w.ys = ys; w.xf = o.xf; w.yf = o.yf; w.ux = o.ux; w.uy = o.uy;
+                w.p = (unsigned)p; w.f = f; w.soft = soft;
+            }
+            qtail += __popc(wm);
+        }
+        // segmented sum over runs of equal triangle; a level runs only when some run spans it
+        {
+            const int key = stays ? f : -1;
+            long long v[3];
+#pragma unroll
+            for (int m = 0; m < 3; ++m) v[m] = stays ? o.v[m] : 0;
+            const int kn = __shfl_down_sync(full, key, 1);
+            const unsigned tails = __ballot_sync(full, (lane == 31) || (kn != key));
+            const int seg_end = lane + __ffs(tails >> lane) - 1;
+            const int kp = __shfl_up_sync(full, key, 1);
+            const bool head = (lane == 0) || (kp != key);
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                if (!__any_sync(full, seg_end - lane >= off)) break;
+#pragma unroll
+                for (int m = 0; m < 3; ++m) {
+                    const long long ov = __shfl_down_sync(full, v[m], off);
+                    if (lane + off <= seg_end) v[m] += ov;
+                }
+            }
+            if (head && key >= 0) {
+                const int4 ew = __ldg(reinterpret_cast<const int4 *>(a.topo + f));       // edge words, neighbour 0
+                red_add_u64(a.ifix + (ew.x >> 1), (ew.x & 1) ? -v[0] : v[0]);
+                red_add_u64(a.ifix + (ew.y >> 1), (ew.y & 1) ? -v[1] : v[1]);
+                red_add_u64(a.ifix + (ew.z >> 1), (ew.z & 1) ? -v[2] : v[2]);
+            }
+        }
+        if (live) { a.ux[p] = o.ux; a.uy[p] = o.uy; }
+        if (stays) {
+            a.x[p] = o.xf; a.y[p] = o.yf;
+            if (a.rec_cap > 0) a.rec_cnt[S->off + a.id[p]] = 0;
+        }
+        if (qtail - qhead >= 32) {
+            __syncwarp();
+            walk64_any(a, q + ((qhead + lane) & (RING64 - 1)));
+            qhead += 32;
+            __syncwarp();
+        }
     }
+    if (qtail > qhead) {
+        __syncwarp();
+        if ((unsigned)lane < qtail - qhead) walk64_any(a, q + ((qhead + lane) & (RING64 - 1)));
+    }
+}
+
+template <int PUSHER>
+static void launch_p64(cudaStream_t st, const StepArgs64 &a)
+{
+    static int per_sm = 0, sms = 0, dev = -1, blk = 0;
+    const size_t ring = (size_t)(a.block / 32) * RING64 * sizeof(Walk64);
+    int d = 0;
+    cudaGetDevice(&d);
+    if (d != dev || blk != a.block) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_particles64<PUSHER>, a.block, ring);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
+        dev = d; blk = a.block;
+        if (per_sm < 1) per_sm = 1;
+    }
+    const long long nw = a.block / 32, need = (a.nchunks + nw - 1) / nw;
+    const long long grid = need < (long long)per_sm * sms ? need : (long long)per_sm * sms;
+    k_particles64<PUSHER><<<(unsigned)grid, a.block, ring, st>>>(a);
 }
 
 void launch_particles64(cudaStream_t st, int pusher, const StepArgs64 &a)
 {
-    if (a.nblocks <= 0) return;
-    const dim3 grid((unsigned)a.nblocks), block(a.block);
+    if (a.nchunks <= 0) return;
     switch (pusher) {
-    case FETDPIC_BORIS: k_particles64<FETDPIC_BORIS><<<grid, block, 0, st>>>(a); break;
-    case FETDPIC_BORIS_TAN: k_particles64<FETDPIC_BORIS_TAN><<<grid, block, 0, st>>>(a); break;
-    case FETDPIC_VAY: k_particles64<FETDPIC_VAY><<<grid, block, 0, st>>>(a); break;
-    default: k_particles64<FETDPIC_HC><<<grid, block, 0, st>>>(a); break;
+    case FETDPIC_BORIS: launch_p64<FETDPIC_BORIS>(st, a); break;
+    case FETDPIC_BORIS_TAN: launch_p64<FETDPIC_BORIS_TAN>(st, a); break;
+    case FETDPIC_VAY: launch_p64<FETDPIC_VAY>(st, a); break;
+    default: launch_p64<FETDPIC_HC>(st, a); break;
     }
 }
 
