@@ -257,54 +257,51 @@ __device__ __forceinline__ F2 rcp_f2(const F2 &x)
 // caller variable needs an address.  Returns (u_x, u_y, v_x, v_y) in units of c.
 struct PushOut { float ux, uy, vx, vy; };
 
-// The same in FP64, for what double-float cannot hold: gamma^2 whose square
-// leaves the FP32 range, |beta|^2 close to gamma^2 (sigma cancels), a Boris-tan
-// angle beyond the series.  Inlined into push_f2, where a nested call would
-// cost the particle kernels spills (24 bytes in the Vay kernel at 72 registers);
-// out of line for Boris-tan, whose FP64 tangent costs more than the call.
+// The same in FP64, for what double-float cannot hold.
 template <int PUSHER>
-__device__ __forceinline__ PushOut push_fp64_inl(float ux, float uy, float ex, float ey, float bz)
+__device__ __noinline__ PushOut push_fp64(float ux, float uy, float ex, float ey, float bz)
 {
     double dux = ux, duy = uy;
     const double dig = push_c1<PUSHER, double, true>(dux, duy, (double)ex, (double)ey, (double)bz);
     return PushOut{(float)dux, (float)duy, (float)(dux * dig), (float)(duy * dig)};
 }
+
+// Whether the double-float push takes a particle with gamma^2 = g2: gamma^4 in
+// the FP32 range, the kick and |beta| below gamma / 8 (sigma then stays above
+// gamma^2 / 4, no cancellation) and, for Boris-tan, the angle within its series.
+// Decided by the caller: with the FP64 form inside push_f2 the 72-register Vay
+// kernel spilled 16 bytes (variant 19 alone 146.8 us a step of the 8 M-particle
+// plasma against 134.9).
 template <int PUSHER>
-__device__ __noinline__ PushOut push_fp64_call(float ux, float uy, float ex, float ey, float bz)
+__device__ __forceinline__ bool f2_takes(float g2, float ex, float ey, float bz)
 {
-    return push_fp64_inl<PUSHER>(ux, uy, ex, ey, bz);
-}
-template <int PUSHER>
-__device__ __forceinline__ PushOut push_fp64(float ux, float uy, float ex, float ey, float bz)
-{
-    if constexpr (PUSHER == FETDPIC_BORIS_TAN) return push_fp64_call<PUSHER>(ux, uy, ex, ey, bz);
-    else return push_fp64_inl<PUSHER>(ux, uy, ex, ey, bz);
+    const float k = PUSHER == FETDPIC_BORIS_TAN ? 1000.f : 64.f;
+    return g2 < 1e17f && k * (bz * bz) < g2 && 64.f * (ex * ex + ey * ey) < g2;
 }
 
 template <int PUSHER>
 __device__ __noinline__ PushOut push_f2(float ux, float uy, float ex, float ey, float bz)
 {
-    const F2 bb = two_prod(bz, bz);
-    const F2 umx = two_sum(ux, ex), umy = two_sum(uy, ey);             // u^-
-    const F2 g2 = sqr(umx) + sqr(umy) + 1.f;
-    if (!(g2.h < 1e18f) || !(4.f * bb.h < g2.h)) return push_fp64<PUSHER>(ux, uy, ex, ey, bz);
     F2 x, y, ig;                                                       // u^{n+1/2}, 1/gamma^{n+1/2}
     if (PUSHER == FETDPIC_VAY) {
         const F2 ig0 = rsqrt_f2(two_prod(ux, ux) + two_prod(uy, uy) + 1.f);
-        const F2 upx = umx + ex + ig0 * uy * bz;
-        const F2 upy = umy + ey - ig0 * ux * bz;
+        const F2 upx = two_sum(ux, ex) + ex + ig0 * uy * bz;
+        const F2 upy = two_sum(uy, ey) + ey - ig0 * ux * bz;
+        const F2 bb = two_prod(bz, bz);
         const F2 sigma = sqr(upx) + sqr(upy) + 1.f - bb;
         const F2 r2 = sqr(sigma) + F2(4.f * bb.h, 4.f * bb.l);
         const F2 s2 = sigma + r2 * rsqrt_f2(r2);
-        if (!(sigma.h > 0.f) || !(s2.h < 4e18f)) return push_fp64<PUSHER>(ux, uy, ex, ey, bz);
         ig = rsqrt_f2(F2(0.5f * s2.h, 0.5f * s2.l));
         const F2 tz = ig * bz;
         const F2 s = rcp_f2(sqr(tz) + 1.f);
         x = s * (upx + upy * tz);
         y = s * (upy - upx * tz);
     } else {
+        const F2 umx = two_sum(ux, ex), umy = two_sum(uy, ey);         // u^-
+        const F2 g2 = sqr(umx) + sqr(umy) + 1.f;
         F2 tz;
         if (PUSHER == FETDPIC_HC) {
+            const F2 bb = two_prod(bz, bz);
             const F2 sigma = g2 - bb;
             const F2 r2 = sqr(sigma) + F2(4.f * bb.h, 4.f * bb.l);
             const F2 s2 = sigma + r2 * rsqrt_f2(r2);
@@ -314,7 +311,6 @@ __device__ __noinline__ PushOut push_f2(float ux, float uy, float ex, float ey, 
             if (PUSHER == FETDPIC_BORIS_TAN) {
                 // tan t = t + t (t^2/3 + 2 t^4/15 + 17 t^6/315 + 62 t^8/2835 + ...): the first
                 // neglected term is below 1e-15 of t for |t| < 0.04
-                if (!(fabsf(tz.h) < 0.04f)) return push_fp64<PUSHER>(ux, uy, ex, ey, bz);
                 const F2 q = sqr(tz);
                 const float r = q.h * q.h * (2.f / 15.f + q.h * (17.f / 315.f + q.h * (62.f / 2835.f)));
                 // 1/3 as a double-float: 1/3 rounded to FP32, and the rest
@@ -622,8 +618,10 @@ __device__ __forceinline__ POne one_particle(float kappa, float wfix, int f, flo
     const float ey = kappa * (l0 * r.r0.y + l1 * r.r0.w + l2 * r.r1.y);
     const float bz = kappa * r.r1.z;
     float vx, vy;
-    if (1.f + ux * ux + uy * uy > 100.f) {
-        const PushOut q = push_f2<PUSHER>(ux, uy, ex, ey, bz);
+    const float gg = 1.f + ux * ux + uy * uy;
+    if (gg > 100.f) {
+        const PushOut q = f2_takes<PUSHER>(gg, ex, ey, bz) ? push_f2<PUSHER>(ux, uy, ex, ey, bz)
+                                                           : push_fp64<PUSHER>(ux, uy, ex, ey, bz);
         ux = q.ux; uy = q.uy; vx = q.vx; vy = q.vy;
     } else {
         const float ig = push_c1<PUSHER, float>(ux, uy, ex, ey, bz);
@@ -645,10 +643,9 @@ __device__ __forceinline__ POne one_particle(float kappa, float wfix, int f, flo
     return o;
 }
 
-__device__ __forceinline__ WalkItem walk_item(unsigned p, int f, int sp, float l0, float l1, const POne &o)
+__device__ __forceinline__ WalkItem walk_item(unsigned p, int f, float l0, float l1, const POne &o)
 {
     WalkItem it;
-    (void)sp;
     it.p = p; it.f = f;
     it.l0 = l0; it.l1 = l1;
     it.ux = o.ux; it.uy = o.uy; it.vx = o.vx; it.vy = o.vy;
@@ -713,7 +710,7 @@ __device__ __forceinline__ void process_chunk(const StepArgs32 &a, unsigned c, i
     if (o.bad) atomicOr(a.status, (unsigned)ST_NONFINITE);
     {
         const unsigned slot = ring_slot(qtail, o.walking, lane);
-        if (o.walking) q[slot & (P32_QUEUE - 1)] = walk_item(p, s.f, s.sp, s.l0, s.l1, o);
+        if (o.walking) q[slot & (P32_QUEUE - 1)] = walk_item(p, s.f, s.l0, s.l1, o);
     }
     {
         const int ew[3] = {__float_as_int(r.r1.w), __float_as_int(r.c1.x), __float_as_int(r.c1.y)};
@@ -808,7 +805,7 @@ __device__ __forceinline__ PState2 load_state2(const StepArgs32 &a, unsigned c, 
 template <int PUSHER, bool SEQ, int WT>
 __device__ __forceinline__ void process_chunk2(const StepArgs32 &a, unsigned c, int lane, const PState2 &s,
                                                const PRec &ra, const PRec &rb_in, WalkItem *q, unsigned &qhead,
-                                               unsigned &qtail, bool &bad, const DepWin &dw)
+                                               unsigned &qtail, const DepWin &dw)
 {
     const unsigned full = 0xffffffffu;
     const unsigned pa = c * 64u + 2u * (unsigned)lane;
@@ -817,7 +814,7 @@ __device__ __forceinline__ void process_chunk2(const StepArgs32 &a, unsigned c, 
     const POne A = one_particle<PUSHER>(kw.x, kw.y, s.fa, s.l0.x, s.l1.x, s.ux.x, s.uy.x, ra);
     {
         const unsigned slot = ring_slot(qtail, A.walking, lane);
-        if (A.walking) q[slot & (P32_QUEUE2 - 1)] = walk_item(pa, s.fa, s.sp, s.l0.x, s.l1.x, A);
+        if (A.walking) q[slot & (P32_QUEUE2 - 1)] = walk_item(pa, s.fa, s.l0.x, s.l1.x, A);
     }
     const int ewa[3] = {__float_as_int(ra.r1.w), __float_as_int(ra.c1.x), __float_as_int(ra.c1.y)};
     PRec rb;
@@ -830,9 +827,9 @@ __device__ __forceinline__ void process_chunk2(const StepArgs32 &a, unsigned c, 
     const POne B = one_particle<PUSHER>(kw.x, kw.y, s.fb, s.l0.y, s.l1.y, s.ux.y, s.uy.y, rb);
     {
         const unsigned slot = ring_slot(qtail, B.walking, lane);
-        if (B.walking) q[slot & (P32_QUEUE2 - 1)] = walk_item(pa + 1, s.fb, s.sp, s.l0.y, s.l1.y, B);
+        if (B.walking) q[slot & (P32_QUEUE2 - 1)] = walk_item(pa + 1, s.fb, s.l0.y, s.l1.y, B);
     }
-    bad |= A.bad | B.bad;
+    if (A.bad || B.bad) atomicOr(a.status, (unsigned)ST_NONFINITE);
     // current of the particles that stay, Eq. (I.assign).  The run of a
     // thread's second particle is reduced across the warp; a first particle that ends a
     // different run (an "orphan") is handed to the previous thread when that thread's second
@@ -919,16 +916,14 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_particles32x2(StepArgs32 a)
     // first state load and the window set-up go ahead of the wait.
     pdl_begin();
     if (c < cend) {
-        bool bad = false;
         for (; c < cend; ++c) {
             const PState2 s = sn;
             if (c + 1 < cend) sn = load_state2(a, c + 1, lane);
             const PRec ra = load_rec(a, s.fa);
             PRec rb;
             if (!SEQ) rb = load_rec(a, s.fb);
-            process_chunk2<PUSHER, SEQ, WT>(a, c, lane, s, ra, rb, q, qhead, qtail, bad, dw);
+            process_chunk2<PUSHER, SEQ, WT>(a, c, lane, s, ra, rb, q, qhead, qtail, dw);
         }
-        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.status, (unsigned)ST_NONFINITE);
         drain<P32_QUEUE2>(a, q, qhead, qtail, lane);
     }
     if constexpr (WT > 0) {
