@@ -92,6 +92,8 @@ struct fetdpic_ctx {
     double2 *extw = nullptr;                 // NULL until a profile is set
     int *face_inst = nullptr;                // FP32: instance of each triangle
     int *tri_c2i = nullptr;                  // [cell_off + caller index] -> stored instance-local index
+    int *edge_c2i = nullptr;                  // [edge_off + caller index] -> stored instance-local index
+    double *field_out = nullptr;              // one instance's e, b, j in the caller's order (reads)
     int *tri_i2c = nullptr;                  // [stored global index] -> caller's instance-local index
     bool ext_on = false;                     // FP32: fold applied fields into the field record
     int *hist = nullptr, *hoff = nullptr, *scan_tmp = nullptr; long long hist_n = 0;
@@ -340,7 +342,7 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
             G.pad = 0;
             Topo &T = tp[co + f];
             for (int m = 0; m < 3; ++m) {
-                const int eg = eo + M.tedge[3 * f + m];
+                const int eg = eo + M.einv[M.tedge[3 * f + m]];
                 T.ew[m] = (eg << 1) | (M.tsign[3 * f + m] < 0 ? 1 : 0);
                 T.nb[m] = M.tnb[3 * f + m] < 0 ? -1 : (((co + M.tnb[3 * f + m]) << 2) | M.tnbm[3 * f + m]);
                 T.node[m] = no + M.rep[M.tri[3 * f + m]];
@@ -360,23 +362,29 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
             }
         }
         for (int e = 0; e < M.ne; ++e) {
-            if (!M.pec[e]) e0[eo + e] = I.e0x * M.evec[2 * e] + I.e0y * M.evec[2 * e + 1];
-            efac[eo + e] = make_int2(co + M.efac[2 * e], M.efac[2 * e + 1] < 0 ? -1 : co + M.efac[2 * e + 1]);
+            const int i = eo + M.einv[e];
+            if (!M.pec[e]) e0[i] = I.e0x * M.evec[2 * e] + I.e0y * M.evec[2 * e + 1];
+            efac[i] = make_int2(co + M.efac[2 * e], M.efac[2 * e + 1] < 0 ? -1 : co + M.efac[2 * e + 1]);
             const double h0 = 1.0 / (P.mu0 * (0.5 * M.d2A[M.efac[2 * e]]));
             const double h1 = M.efac[2 * e + 1] < 0 ? 0.0 : 1.0 / (P.mu0 * (0.5 * M.d2A[M.efac[2 * e + 1]]));
-            ecoef[eo + e] = make_double2(M.efsign[2 * e] * h0, M.efsign[2 * e + 1] * h1);
-            einst[eo + e] = k;
+            ecoef[i] = make_double2(M.efsign[2 * e] * h0, M.efsign[2 * e + 1] * h1);
+            einst[i] = k;
         }
         // d^0 = [*eps] e^0 over all edges
         for (int e = 0; e < M.ne; ++e) {
             double s = 0.0;
-            for (long long q = M.h_rp[e]; q < M.h_rp[e + 1]; ++q) s += M.h_v[q] * e0[eo + M.h_ci[q]];
-            d0[eo + e] = s;
+            for (long long q = M.h_rp[e]; q < M.h_rp[e + 1]; ++q) s += M.h_v[q] * e0[eo + M.einv[M.h_ci[q]]];
+            d0[eo + M.einv[e]] = s;
         }
-        for (size_t a = 0; a < M.free_edges.size(); ++a) {
-            mrow.push_back(eo + M.free_edges[a]);
+        // rows in stored edge order, a row's entries in the caller's (the order of its sum)
+        std::vector<int> fidx(M.ne, -1);
+        for (size_t a = 0; a < M.free_edges.size(); ++a) fidx[M.free_edges[a]] = (int)a;
+        for (int i = 0; i < M.ne; ++i) {
+            const int a = fidx[M.eperm[i]];
+            if (a < 0) continue;
+            mrow.push_back(eo + i);
             for (long long q = M.m_rp[a]; q < M.m_rp[a + 1]; ++q) {
-                mci.push_back(eo + M.m_ci[q]);
+                mci.push_back(eo + M.einv[M.m_ci[q]]);
                 mv.push_back(I.dt * M.m_v[q]);
             }
             mrp.push_back((long long)mci.size());
@@ -443,7 +451,7 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         for (int k = 0; k < n_inst; ++k) {
             const HostMesh &M = ctx->mesh[k];
             for (int e = 0; e < M.ne; ++e) {
-                const int eg = ctx->edge_off[k] + e;
+                const int eg = ctx->edge_off[k] + M.einv[e];
                 nedge[fill[ctx->node_off[k] + M.edge[2 * e]]++] = eg << 1;            // leaves the node: +1
                 nedge[fill[ctx->node_off[k] + M.edge[2 * e + 1]]++] = (eg << 1) | 1;  // enters the node: -1
             }
@@ -451,8 +459,8 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         for (int k = 0; k < n_inst; ++k) {
             const HostMesh &M = ctx->mesh[k];
             const int eo = ctx->edge_off[k];
-            for (int e = 0; e < M.ne; ++e) {
-                for (long long q = M.h_rp[e]; q < M.h_rp[e + 1]; ++q) { hci.push_back(eo + M.h_ci[q]); hv.push_back(M.h_v[q]); }
+            for (int e : M.eperm) {
+                for (long long q = M.h_rp[e]; q < M.h_rp[e + 1]; ++q) { hci.push_back(eo + M.einv[M.h_ci[q]]); hv.push_back(M.h_v[q]); }
                 hrp.push_back((long long)hci.size());
             }
         }
@@ -486,6 +494,10 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         }
         ctx->tri_c2i = ctx->alloc<int>(ctx->F);
         ctx->tri_i2c = ctx->alloc<int>(ctx->F);
+        ctx->edge_c2i = ctx->alloc<int>(ctx->E);
+        size_t most = 0;
+        for (const HostMesh &M : ctx->mesh) most = std::max(most, 2 * (size_t)M.ne + M.nf);
+        ctx->field_out = ctx->alloc<double>(most);
         ctx->ext_dev = ctx->alloc<ExtField>(n_inst);
         ctx->ext_amp = ctx->alloc<double>(n_inst);
         if (P.precision == FETDPIC_FP32) ctx->face_inst = ctx->alloc<int>(ctx->F);
@@ -564,16 +576,18 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         }
     }
     {
-        std::vector<int> c2i(ctx->F), i2c(ctx->F);
+        std::vector<int> c2i(ctx->F), i2c(ctx->F), ec2i(ctx->E);
         for (int k = 0; k < n_inst; ++k) {
             const HostMesh &M = ctx->mesh[k];
             for (int f = 0; f < M.nf; ++f) {
                 c2i[ctx->cell_off[k] + f] = M.inv[f];
                 i2c[ctx->cell_off[k] + f] = M.perm[f];
             }
+            std::copy(M.einv.begin(), M.einv.end(), ec2i.begin() + ctx->edge_off[k]);
         }
         rc = rc ? rc : upload(ctx, ctx->tri_c2i, c2i.data(), c2i.size());
         rc = rc ? rc : upload(ctx, ctx->tri_i2c, i2c.data(), i2c.size());
+        rc = rc ? rc : upload(ctx, ctx->edge_c2i, ec2i.data(), ec2i.size());
     }
     rc = rc ? rc : upload(ctx, ctx->m_soff, soff.data(), soff.size());
     ctx->m_entries = soff.back();
@@ -1213,6 +1227,25 @@ extern "C" int fetdpic_write_particles(fetdpic_ctx *ctx, int species, const doub
     return FETDPIC_OK;
 }
 
+// Edge unknowns of an instance (caller's order, 0 on PEC edges) to the device, with the dual flux
+// restarted consistently: d = [*eps] e.  Waits for the copies.
+static int upload_edges(fetdpic_ctx *ctx, int inst, const std::vector<double> &ev)
+{
+    const HostMesh &M = ctx->mesh[inst];
+    std::vector<double> es(M.ne), ds(M.ne);
+    for (int k = 0; k < M.ne; ++k) {
+        double s = 0.0;
+        for (long long q = M.h_rp[k]; q < M.h_rp[k + 1]; ++q) s += M.h_v[q] * ev[M.h_ci[q]];
+        es[M.einv[k]] = ev[k];
+        ds[M.einv[k]] = s;
+    }
+    int rc = upload(ctx, ctx->e + ctx->edge_off[inst], es.data(), es.size());
+    rc = rc ? rc : upload(ctx, ctx->d + ctx->edge_off[inst], ds.data(), ds.size());
+    if (rc) return rc;
+    CK(cudaStreamSynchronize(ctx->stream));
+    return FETDPIC_OK;
+}
+
 extern "C" int fetdpic_write_fields(fetdpic_ctx *ctx, int inst, const double *e, const double *b)
 {
     if (!ctx || inst < 0 || inst >= (int)ctx->mesh.size()) return FETDPIC_EINVAL;
@@ -1220,15 +1253,8 @@ extern "C" int fetdpic_write_fields(fetdpic_ctx *ctx, int inst, const double *e,
     if (e) {
         std::vector<double> ev(e, e + M.ne);
         for (int k = 0; k < M.ne; ++k) if (M.pec[k]) ev[k] = 0.0;
-        int rc = upload(ctx, ctx->e + ctx->edge_off[inst], ev.data(), ev.size());
+        int rc = upload_edges(ctx, inst, ev);
         if (rc) return rc;
-        // restart the dual flux consistently: d = [*eps] e
-        std::vector<double> dv(M.ne, 0.0);
-        for (int k = 0; k < M.ne; ++k)
-            for (long long q = M.h_rp[k]; q < M.h_rp[k + 1]; ++q) dv[k] += M.h_v[q] * ev[M.h_ci[q]];
-        rc = upload(ctx, ctx->d + ctx->edge_off[inst], dv.data(), dv.size());
-        if (rc) return rc;
-        CK(cudaStreamSynchronize(ctx->stream));
     }
     if (b) {
         std::vector<double> bs(M.nf);                // stored triangle order
@@ -1268,17 +1294,11 @@ extern "C" int fetdpic_solve_electrostatic(fetdpic_ctx *ctx, int inst, int *iter
     if (rc) return ctx->fail(rc, msg);
     CK(cudaSetDevice(ctx->device));
     CK(cudaStreamSynchronize(ctx->stream));
-    std::vector<double> ev(M.ne);
-    CK(cudaMemcpy(ev.data(), ctx->e + ctx->edge_off[inst], sizeof(double) * M.ne, cudaMemcpyDeviceToHost));
-    for (int k = 0; k < M.ne; ++k) ev[k] += de[k];
-    rc = upload(ctx, ctx->e + ctx->edge_off[inst], ev.data(), ev.size());
+    std::vector<double> es(M.ne), ev(M.ne);
+    CK(cudaMemcpy(es.data(), ctx->e + ctx->edge_off[inst], sizeof(double) * M.ne, cudaMemcpyDeviceToHost));
+    for (int k = 0; k < M.ne; ++k) ev[k] = es[M.einv[k]] + de[k];
+    rc = upload_edges(ctx, inst, ev);
     if (rc) return rc;
-    std::vector<double> dv(M.ne, 0.0);
-    for (int k = 0; k < M.ne; ++k)
-        for (long long p = M.h_rp[k]; p < M.h_rp[k + 1]; ++p) dv[k] += M.h_v[p] * ev[M.h_ci[p]];
-    rc = upload(ctx, ctx->d + ctx->edge_off[inst], dv.data(), dv.size());
-    if (rc) return rc;
-    CK(cudaStreamSynchronize(ctx->stream));
     ctx->gauss_abs[inst] = 1;
     auto &an = ctx->abs_nodes[inst];
     an.assign(M.nn, 0);
@@ -1300,14 +1320,21 @@ extern "C" int fetdpic_read(fetdpic_ctx *ctx, int inst, double *e, double *b, do
                             int species, double *x, double *u, int *cell)
 {
     if (!ctx || inst < 0 || inst >= (int)ctx->mesh.size()) return FETDPIC_EINVAL;
-    CK(cudaStreamSynchronize(ctx->stream));
     const HostMesh &M = ctx->mesh[inst];
-    if (e) CK(cudaMemcpyAsync(e, ctx->e + ctx->edge_off[inst], sizeof(double) * M.ne, cudaMemcpyDeviceToHost, ctx->stream));
-    std::vector<double> bs(b ? M.nf : 0);
-    if (b) CK(cudaMemcpyAsync(bs.data(), ctx->b + ctx->cell_off[inst], sizeof(double) * M.nf, cudaMemcpyDeviceToHost, ctx->stream));
-    if (j) CK(cudaMemcpyAsync(j, ctx->j + ctx->edge_off[inst], sizeof(double) * M.ne, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaSetDevice(ctx->device));
+    {
+        // to the caller's edge and triangle order on the device, then to the host
+        const int eo = ctx->edge_off[inst], co = ctx->cell_off[inst];
+        double *oe = ctx->field_out, *oj = oe + M.ne, *ob = oj + M.ne;
+        if (e) launch_gather_field(ctx->stream, M.ne, eo, ctx->edge_c2i, ctx->e, oe);
+        if (b) launch_gather_field(ctx->stream, M.nf, co, ctx->tri_c2i, ctx->b, ob);
+        if (j) launch_gather_field(ctx->stream, M.ne, eo, ctx->edge_c2i, ctx->j, oj);
+        CK(cudaGetLastError());
+        if (e) CK(cudaMemcpyAsync(e, oe, sizeof(double) * M.ne, cudaMemcpyDeviceToHost, ctx->stream));
+        if (b) CK(cudaMemcpyAsync(b, ob, sizeof(double) * M.nf, cudaMemcpyDeviceToHost, ctx->stream));
+        if (j) CK(cudaMemcpyAsync(j, oj, sizeof(double) * M.ne, cudaMemcpyDeviceToHost, ctx->stream));
+    }
     CK(cudaStreamSynchronize(ctx->stream));
-    if (b) for (int f = 0; f < M.nf; ++f) b[M.perm[f]] = bs[f];   // back to the caller's triangle order
     if (x || u || cell) {
         int rc = finalize(ctx);
         if (rc) return rc;
@@ -1433,6 +1460,13 @@ extern "C" int fetdpic_read_walk(fetdpic_ctx *ctx, int species, int *cnt, int *r
     CK(cudaStreamSynchronize(ctx->stream));
     CK(cudaMemcpy(cnt, ctx->rec_cnt + D.off, sizeof(int) * D.n, cudaMemcpyDeviceToHost));
     CK(cudaMemcpy(rec, ctx->rec + D.off * rc_, sizeof(int) * D.n * rc_, cudaMemcpyDeviceToHost));
+    // the kernels record stored edge ids; entries beyond a particle's count are not set
+    const HostMesh &M = ctx->mesh[D.inst];
+    for (long long k = 0; k < D.n; ++k)
+        for (int c = 0; c < std::min<int>(cnt[k], (int)rc_); ++c) {
+            int &v = rec[k * (long long)rc_ + c];
+            v = v >= 0 ? M.eperm[v] : -(M.eperm[-v - 1] + 1);
+        }
     return FETDPIC_OK;
 }
 
@@ -1525,7 +1559,7 @@ extern "C" int fetdpic_set_probes(fetdpic_ctx *ctx, long long n, const int *inst
             const double sg = M.tsign[3 * f + m];
             W.w[2 * m] = sg * (l[a] * M.gx[3 * f + b] - l[b] * M.gx[3 * f + a]);
             W.w[2 * m + 1] = sg * (l[a] * M.gy[3 * f + b] - l[b] * M.gy[3 * f + a]);
-            W.eg[m] = ctx->edge_off[k] + M.tedge[3 * f + m];
+            W.eg[m] = ctx->edge_off[k] + M.einv[M.tedge[3 * f + m]];
         }
         W.pad = 0;
     }

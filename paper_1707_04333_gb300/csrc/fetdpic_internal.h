@@ -45,6 +45,10 @@ struct HostMesh {
     // triangle order: the library stores triangles along a Hilbert curve of their centroids;
     // perm[internal] = the caller's index, inv[caller] = internal index
     std::vector<int> perm, inv;
+    // edges are stored in the order in which the stored triangles first touch them:
+    // eperm[internal] = the caller's edge, einv[caller] = internal (everything else in
+    // this struct numbers edges as the caller does)
+    std::vector<int> eperm, einv;
 };
 
 // Order of the triangles along a Hilbert curve of their centroids (ties by
@@ -311,6 +315,9 @@ void launch_ingest(cudaStream_t st, long long n, long long cap, long long off, i
 // to the caller's instance-local index.  A slot with triangle -1 and a load
 // index in [0, n) is a particle dropped by a write: its entry gets NaN
 // position and momentum and triangle -1.
+// dst[k] = src[off + c2i[off + k]]: one instance's edge or triangle values in the caller's order.
+void launch_gather_field(cudaStream_t st, int n, int off, const int *c2i, const double *src, double *dst);
+
 void launch_unsort64(cudaStream_t st, long long n, const int *cell, const int *id, const double *x,
                      const double *y, const double *ux, const double *uy, long long off, long long cap,
                      const int *i2c, double *ox, double *ou, int *oc);

@@ -450,6 +450,18 @@ void launch_ingest(cudaStream_t st, long long n, long long cap, long long off, i
                                                             geo, inv_c, cell_o, id_o, f0, f1, f2, f3, status);
 }
 
+__global__ void __launch_bounds__(256) k_gather_field(int n, int off, const int *__restrict__ c2i,
+                                                      const double *__restrict__ src, double *__restrict__ dst)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) dst[k] = src[off + c2i[off + k]];
+}
+
+void launch_gather_field(cudaStream_t st, int n, int off, const int *c2i, const double *src, double *dst)
+{
+    if (n > 0) k_gather_field<<<(n + 255) / 256, 256, 0, st>>>(n, off, c2i, src, dst);
+}
+
 __global__ void k_unsort64(long long off, long long cap, long long n, const int *__restrict__ cell, const int *__restrict__ id,
                            const double *__restrict__ x, const double *__restrict__ y,
                            const double *__restrict__ ux, const double *__restrict__ uy, const int *__restrict__ i2c,

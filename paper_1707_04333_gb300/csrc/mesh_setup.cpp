@@ -178,6 +178,10 @@ int build_mesh(HostMesh &M, int nn, const double *xy, int nf, const int *tri_cal
             msg = "inconsistent orientation across edge " + std::to_string(e); return FETDPIC_EMESH;
         }
     }
+    M.einv.assign(ne, -1);
+    M.eperm.clear(); M.eperm.reserve(ne);
+    for (int e : M.tedge)
+        if (M.einv[e] < 0) { M.einv[e] = (int)M.eperm.size(); M.eperm.push_back(e); }
     M.tshift.assign(3 * (size_t)nf, 0);
     for (int f = 0; f < nf; ++f)
         for (int m = 0; m < 3; ++m) {
