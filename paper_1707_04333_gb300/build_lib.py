@@ -26,10 +26,11 @@ CU_SOURCES = {
     "kernels_fp64.cu": ["-fmad=false"],
     "kernels_fp32.cu": ["-prec-div=false", "-prec-sqrt=false"],
     "kernels_common.cu": [],
+    "kernels_field.cu": [],
     "kernels_check.cu": [],
     "fetdpic_api.cu": [],
 }
-CPP_SOURCES = ["mesh_setup.cpp"]
+CPP_SOURCES = ["mesh_setup.cpp", "field_patches.cpp"]
 
 
 def _nvcc() -> str:

@@ -58,6 +58,12 @@ struct fetdpic_ctx {
     Rec64 *rec64 = nullptr; Rec32 *rec32 = nullptr;
     double *e = nullptr, *b = nullptr, *d = nullptr, *r = nullptr, *j = nullptr;
     unsigned long long *ifix = nullptr;
+    // field update by patches (kernels_field.cu): its tables, and the second buffers that e, b and
+    // the current accumulator go to and from when it carries the next step's Faraday update
+    bool patches = false;
+    FieldArgs field{};
+    double *e_alt = nullptr, *b_alt = nullptr, *e_a = nullptr;     // e_a: the first buffer (parity reference)
+    unsigned long long *ifix_alt = nullptr;
     int2 *efac = nullptr; double2 *ecoef = nullptr; int *einst = nullptr;
     double *inst_unit = nullptr, *inst_dt = nullptr;
     int *edge_off_dev = nullptr;
@@ -128,11 +134,13 @@ struct fetdpic_ctx {
     std::vector<size_t> rd_off;
 
     // captured one-step graphs: [pusher][particle-buffer parity][step sorts][late hybrid step]
-    cudaGraphExec_t graph[4][2][2][2] = {};
-    long long graph_launches[4][2][2][2] = {};
-    // captured sort cycles (sort_interval steps, the last of which sorts): [pusher][parity at the start]
-    cudaGraphExec_t cycle[4][2] = {};
-    long long cycle_launches[4][2] = {};
+    // [field-buffer parity]
+    cudaGraphExec_t graph[4][2][2][2][2] = {};
+    long long graph_launches[4][2][2][2][2] = {};
+    // captured sort cycles (sort_interval steps, the last of which sorts): [pusher][particle-buffer
+    // parity at the start][field-buffer parity]
+    cudaGraphExec_t cycle[4][2][2] = {};
+    long long cycle_launches[4][2][2] = {};
     int *cell_a = nullptr;                    // the first particle buffer (parity reference)
 
     std::vector<void *> allocs;
@@ -150,8 +158,9 @@ struct fetdpic_ctx {
         if (stream) cudaStreamSynchronize(stream);
         if (side) cudaStreamSynchronize(side);
         if (io) cudaStreamSynchronize(io);
-        for (auto &a : graph) for (auto &b : a) for (auto &c : b) for (auto &g : c) if (g) cudaGraphExecDestroy(g);
-        for (auto &a : cycle) for (auto &g : a) if (g) cudaGraphExecDestroy(g);
+        for (auto &a : graph) for (auto &b : a) for (auto &c : b) for (auto &d : c) for (auto &g : d)
+            if (g) cudaGraphExecDestroy(g);
+        for (auto &a : cycle) for (auto &b : a) for (auto &g : b) if (g) cudaGraphExecDestroy(g);
         for (void *q : allocs) {
             if (p.dev_free) p.dev_free(q, p.alloc_user);
             else cudaFree(q);
@@ -403,11 +412,26 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
                 std::copy(M.tshift.begin(), M.tshift.end(), tsh.begin() + 3 * (size_t)ctx->cell_off[k]);
         }
     ctx->nfree = (long long)mrow.size();
-    // sliced ELL (32 rows per slice, column-major inside a slice)
+    const bool f32 = P.precision == FETDPIC_FP32;
+    // the field update by patches, unless the cooperative form is asked for or a patch's edges do
+    // not fit its block (a dense inverse)
+    PatchSet ps;
+    if (!P.fuse_field_update && P.spai_level >= 0) {
+        std::vector<int> te(3 * (size_t)ctx->F), row(ctx->E, -1);
+        for (int f = 0; f < ctx->F; ++f)
+            for (int m = 0; m < 3; ++m) te[3 * (size_t)f + m] = tp[f].ew[m] >> 1;
+        for (size_t r = 0; r < mrow.size(); ++r) row[mrow[r]] = (int)r;
+        int sms = 0;
+        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+        ps = build_patches(PatchInput{ctx->F, te.data(), row.data(), mrp.data(), mci.data(), mv.data()},
+                           field_patch_size(ctx->F, sms));
+        ctx->patches = ps.ok && field_smem(f32, ps.max_r, ps.max_e) <= FIELD_SMEM_MAX;
+    }
+    // else sliced ELL over all rows (32 rows per slice, column-major inside a slice)
     std::vector<long long> soff(1, 0);
     std::vector<int> sci;
     std::vector<double> sv;
-    {
+    if (!ctx->patches) {
         const long long nr = ctx->nfree;
         for (long long s0 = 0; s0 < nr; s0 += 32) {
             long long wmax = 0;
@@ -427,8 +451,9 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
             soff.push_back(base + 32 * wmax);
         }
     }
+    const std::vector<double> &mat = ctx->patches ? ps.val : sv;
     std::vector<float> sv32;
-    if (P.precision == FETDPIC_FP32) { sv32.resize(sv.size()); for (size_t k = 0; k < sv.size(); ++k) sv32[k] = (float)sv[k]; }
+    if (f32) sv32.assign(mat.begin(), mat.end());
     // node -> edge incidence (fixed order: ascending edge id per node) and the full [*eps]
     std::vector<int> nrp, nedge, ninst(ctx->N);
     std::vector<long long> hrp(1, 0);
@@ -479,7 +504,6 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         ctx->e = ctx->alloc<double>(ctx->E);
         ctx->b = ctx->alloc<double>(ctx->F);
         ctx->d = ctx->alloc<double>(ctx->E);
-        ctx->r = ctx->alloc<double>(ctx->E);
         ctx->j = ctx->alloc<double>(ctx->E);
         ctx->ifix = ctx->alloc<unsigned long long>(ctx->E);
         ctx->efac = ctx->alloc<int2>(ctx->E);
@@ -501,16 +525,37 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         ctx->ext_dev = ctx->alloc<ExtField>(n_inst);
         ctx->ext_amp = ctx->alloc<double>(n_inst);
         if (P.precision == FETDPIC_FP32) ctx->face_inst = ctx->alloc<int>(ctx->F);
-        ctx->m_soff = ctx->alloc<long long>(soff.size());
-        ctx->m_row = ctx->alloc<int>(mrow.size());
-        ctx->m_ci = ctx->alloc<int>(sci.size());
-        if (P.precision == FETDPIC_FP32) {
-            ctx->m_v32 = ctx->alloc<float>(sv32.size());
-            ctx->r32 = ctx->alloc<float>(ctx->E);
-            CK(cudaMemset(ctx->r32, 0, sizeof(float) * ctx->E));     // read by the SPAI product
+        if (f32) ctx->m_v32 = ctx->alloc<float>(mat.size());
+        else ctx->m_v = ctx->alloc<double>(mat.size());
+        if (ctx->patches) {
+            FieldArgs &A = ctx->field;
+            A.patch = ctx->alloc<FieldPatch>(ps.patch.size());
+            A.xlist = ctx->alloc<int>(ps.xlist.size());
+            A.tloc = ctx->alloc<ushort4>(ctx->F);
+            A.row_loc = ctx->alloc<unsigned short>(ps.row_loc.size());
+            A.col = ctx->alloc<unsigned>(ps.col.size() / 2);
+            A.soff = ctx->alloc<long long>(ps.soff.size());
+            ctx->e_alt = ctx->alloc<double>(ctx->E);
+            ctx->b_alt = ctx->alloc<double>(ctx->F);
+            ctx->ifix_alt = ctx->alloc<unsigned long long>(ctx->E);
+            CK(cudaMemset(ctx->e_alt, 0, sizeof(double) * ctx->E));  // PEC edges are 0 in both buffers
+            CK(cudaMemset(ctx->b_alt, 0, sizeof(double) * ctx->F));
+            CK(cudaMemset(ctx->ifix_alt, 0, sizeof(unsigned long long) * ctx->E));
+            A.npatch = (int)ps.patch.size();
+            A.max_r = ps.max_r; A.max_e = ps.max_e; A.T = ps.T;
+            CK(field_setup(field_smem(f32, ps.max_r, ps.max_e)));
         } else {
-            ctx->m_v = ctx->alloc<double>(sv.size());
+            ctx->m_soff = ctx->alloc<long long>(soff.size());
+            ctx->m_row = ctx->alloc<int>(mrow.size());
+            ctx->m_ci = ctx->alloc<int>(sci.size());
+            ctx->r = ctx->alloc<double>(ctx->E);
+            CK(cudaMemset(ctx->r, 0, sizeof(double) * ctx->E));
+            if (f32) {
+                ctx->r32 = ctx->alloc<float>(ctx->E);
+                CK(cudaMemset(ctx->r32, 0, sizeof(float) * ctx->E));     // read by the SPAI product
+            }
         }
+        ctx->e_a = ctx->e;
         ctx->status = ctx->alloc<unsigned>(1);
         ctx->gbar = ctx->alloc<unsigned>(GBAR_WORDS);
         if (ctx->gbar) CK(cudaMemset(ctx->gbar, 0, sizeof(unsigned) * GBAR_WORDS));
@@ -589,16 +634,25 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         rc = rc ? rc : upload(ctx, ctx->tri_i2c, i2c.data(), i2c.size());
         rc = rc ? rc : upload(ctx, ctx->edge_c2i, ec2i.data(), ec2i.size());
     }
-    rc = rc ? rc : upload(ctx, ctx->m_soff, soff.data(), soff.size());
-    ctx->m_entries = soff.back();
-    rc = rc ? rc : upload(ctx, ctx->m_row, mrow.data(), mrow.size());
-    rc = rc ? rc : upload(ctx, ctx->m_ci, sci.data(), sci.size());
-    if (P.precision == FETDPIC_FP32) rc = rc ? rc : upload(ctx, ctx->m_v32, sv32.data(), sv32.size());
-    else rc = rc ? rc : upload(ctx, ctx->m_v, sv.data(), sv.size());
+    if (ctx->patches) {
+        const FieldArgs &A = ctx->field;
+        rc = rc ? rc : upload(ctx, const_cast<FieldPatch *>(A.patch), ps.patch.data(), ps.patch.size());
+        rc = rc ? rc : upload(ctx, const_cast<int *>(A.xlist), ps.xlist.data(), ps.xlist.size());
+        rc = rc ? rc : upload(ctx, (unsigned short *)const_cast<ushort4 *>(A.tloc), ps.tloc.data(), ps.tloc.size());
+        rc = rc ? rc : upload(ctx, const_cast<unsigned short *>(A.row_loc), ps.row_loc.data(), ps.row_loc.size());
+        rc = rc ? rc : upload(ctx, (unsigned short *)const_cast<unsigned *>(A.col), ps.col.data(), ps.col.size());
+        rc = rc ? rc : upload(ctx, const_cast<long long *>(A.soff), ps.soff.data(), ps.soff.size());
+    } else {
+        rc = rc ? rc : upload(ctx, ctx->m_soff, soff.data(), soff.size());
+        ctx->m_entries = soff.back();
+        rc = rc ? rc : upload(ctx, ctx->m_row, mrow.data(), mrow.size());
+        rc = rc ? rc : upload(ctx, ctx->m_ci, sci.data(), sci.size());
+    }
+    if (f32) rc = rc ? rc : upload(ctx, ctx->m_v32, sv32.data(), sv32.size());
+    else rc = rc ? rc : upload(ctx, ctx->m_v, mat.data(), mat.size());
     if (rc) return rc;
     CK(cudaMemsetAsync(ctx->ifix, 0, sizeof(unsigned long long) * ctx->E, ctx->stream));
     CK(cudaMemsetAsync(ctx->j, 0, sizeof(double) * ctx->E, ctx->stream));
-    CK(cudaMemsetAsync(ctx->r, 0, sizeof(double) * ctx->E, ctx->stream));
     CK(cudaMemsetAsync(ctx->status, 0, sizeof(unsigned), ctx->stream));
     ctx->unit_host.assign(n_inst, 0.0);
     ctx->fixscale.assign(n_inst, 1.0);
@@ -954,9 +1008,27 @@ static void do_sort(fetdpic_ctx *ctx, cudaStream_t st)
     for (int k = 0; k < 4; ++k) std::swap(ctx->f[k], ctx->f_tmp[k]);
 }
 
+// The buffers of e, b and the current accumulator change places (a field update
+// that carried the next step's Faraday).
+static void swap_fields(fetdpic_ctx *ctx)
+{
+    std::swap(ctx->e, ctx->e_alt);
+    std::swap(ctx->b, ctx->b_alt);
+    std::swap(ctx->ifix, ctx->ifix_alt);
+}
+
+// Whether the steps of one call may share a field update: Ampere's of one step
+// with Faraday's of the next (no stage events, whose stages are separate, and no
+// checks, which look at the current between them).
+static bool can_merge(const fetdpic_ctx *ctx)
+{
+    return ctx->patches && ctx->p.time_stages == 0 && ctx->p.check_interval <= 0;
+}
+
 // One time step: Faraday (+ field record), particles, Ampere, periodic sort.
-// `timed`: record stage events (time_stages = 1).
-static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed)
+// `timed`: record stage events (time_stages = 1).  `begun`: the previous step's
+// field update carried this step's Faraday; `more`: this step's carries the next's.
+static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool begun = false, bool more = false)
 {
     long long launches = 0;
     const bool f32 = ctx->p.precision == FETDPIC_FP32;
@@ -982,11 +1054,13 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed)
     // stage events need each stage to start after the previous one: no early launch when timed
     A.pdl = !timed;
     if (timed) mark(ctx, -1);
-    if (f32)
-        launch_faraday32(ctx->stream, ctx->F, ctx->csta, ctx->cstb, ctx->dtinv, ctx->e, ctx->b, ctx->rec32,
-                         (float)(0.5 / (ctx->p.c * ctx->p.c)), x, !timed);
-    else launch_faraday64(ctx->stream, ctx->F, ctx->geo64, ctx->topo, ctx->e, ctx->b, ctx->rec64);
-    launches += ctx->F > 0;
+    const float inv2c2 = (float)(0.5 / (ctx->p.c * ctx->p.c));
+    if (begun) {}
+    else if (f32)
+        launch_faraday32(ctx->stream, ctx->F, ctx->csta, ctx->cstb, ctx->dtinv, ctx->e, ctx->b, ctx->rec32, inv2c2, x,
+                         ctx->E, ctx->ifix, !timed);
+    else launch_faraday64(ctx->stream, ctx->F, ctx->geo64, ctx->topo, ctx->e, ctx->b, ctx->rec64, ctx->E, ctx->ifix);
+    launches += ctx->F > 0 && !begun;
     if (timed) mark(ctx, 0);
     if (check && !ctx->q_prev_valid) { charge_now(ctx, ctx->q0); launches += 2; }
     if (ctx->nblocks > 0) {
@@ -1016,8 +1090,27 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed)
         launch_dce(ctx->stream, ctx->N, ctx->nrp, ctx->nedge, ctx->ninst, ctx->ifix, ctx->q0, ctx->q1, ctx->chk_out);
         launches += 3;
     }
-    launch_ampere(ctx->stream, A);
-    launches += A.fused ? (ctx->E > 0 || ctx->nfree > 0) : (ctx->E > 0) + (ctx->nfree > 0);
+    if (ctx->patches) {
+        FieldArgs W = ctx->field;
+        W.v32 = ctx->m_v32; W.v64 = ctx->m_v;
+        W.efac = ctx->efac; W.ecoef = ctx->ecoef; W.einst = ctx->einst;
+        W.inst_unit = ctx->inst_unit; W.inst_dt = ctx->inst_dt;
+        W.b = ctx->b; W.ifix = ctx->ifix; W.j = ctx->j; W.d = A.d;
+        W.e = ctx->e; W.e_next = more ? ctx->e_alt : ctx->e;
+        W.one_inst = ctx->mesh.size() == 1;
+        W.early = ctx->nblocks > 0;
+        W.pdl = !timed;
+        W.faraday = more;
+        W.b_next = ctx->b_alt; W.ifix_next = ctx->ifix_alt;
+        W.csta = ctx->csta; W.cstb = ctx->cstb; W.dtinv = ctx->dtinv; W.rec32 = ctx->rec32; W.inv2c2 = inv2c2; W.ext = x;
+        W.geo = ctx->geo64; W.topo = ctx->topo; W.rec64 = ctx->rec64;
+        launch_field(ctx->stream, W);
+        ++launches;
+        if (more) swap_fields(ctx);
+    } else {
+        launch_ampere(ctx->stream, A);
+        launches += A.fused ? (ctx->E > 0 || ctx->nfree > 0) : (ctx->E > 0) + (ctx->nfree > 0);
+    }
     if (ctx->probe_n > 0) {
         launch_probe(ctx->stream, ctx->probe_n, ctx->probe_w, ctx->e, ctx->probe_ring, ctx->probe_cap,
                      ctx->probe_count);
@@ -1058,7 +1151,8 @@ static int graph_step(fetdpic_ctx *ctx, int pusher, long long &launches)
     const int parity = ctx->cell == ctx->cell_a ? 0 : 1;
     const Hybrid *hy = hybrid_of(ctx->p.kernel_variant);
     const int late = ctx->p.precision == FETDPIC_FP32 && hy && step_variant(ctx) == hy->late ? 1 : 0;
-    cudaGraphExec_t &g = ctx->graph[pusher][parity][sorts ? 1 : 0][late];
+    const int fields = ctx->e == ctx->e_a ? 0 : 1;
+    cudaGraphExec_t &g = ctx->graph[pusher][parity][sorts ? 1 : 0][late][fields];
     if (!g) {
         cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
@@ -1068,13 +1162,13 @@ static int graph_step(fetdpic_ctx *ctx, int pusher, long long &launches)
         e = cudaGraphInstantiate(&g, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) { g = nullptr; return ctx->cuda_fail(e, "cudaGraphInstantiate"); }
-        ctx->graph_launches[pusher][parity][sorts ? 1 : 0][late] = n;
+        ctx->graph_launches[pusher][parity][sorts ? 1 : 0][late][fields] = n;
         CK(cudaGraphLaunch(g, ctx->stream));
         launches += n;
         return FETDPIC_OK;
     }
     CK(cudaGraphLaunch(g, ctx->stream));
-    launches += ctx->graph_launches[pusher][parity][sorts ? 1 : 0][late];
+    launches += ctx->graph_launches[pusher][parity][sorts ? 1 : 0][late][fields];
     // host-side effects of the step the graph replays
     ++ctx->steps_done;
     ctx->q_prev_valid = false;
@@ -1095,25 +1189,28 @@ static int cycle_step(fetdpic_ctx *ctx, int pusher, long long &launches)
 {
     const int parity = ctx->cell == ctx->cell_a ? 0 : 1;
     const int L = ctx->p.sort_interval;
-    cudaGraphExec_t &g = ctx->cycle[pusher][parity];
+    const int fields = ctx->e == ctx->e_a ? 0 : 1;
+    const bool merge = can_merge(ctx);
+    cudaGraphExec_t &g = ctx->cycle[pusher][parity][fields];
     if (!g) {
         cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
         long long n = 0;
-        for (int k = 0; k < L; ++k) n += enqueue_step(ctx, pusher, false);
+        for (int k = 0; k < L; ++k) n += enqueue_step(ctx, pusher, false, merge && k > 0, merge && k + 1 < L);
         cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
         if (e != cudaSuccess) return ctx->cuda_fail(e, "cudaStreamEndCapture");
         e = cudaGraphInstantiate(&g, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) { g = nullptr; return ctx->cuda_fail(e, "cudaGraphInstantiate"); }
-        ctx->cycle_launches[pusher][parity] = n;
+        ctx->cycle_launches[pusher][parity][fields] = n;
         CK(cudaGraphLaunch(g, ctx->stream));
         launches += n;
         return FETDPIC_OK;
     }
     CK(cudaGraphLaunch(g, ctx->stream));
-    launches += ctx->cycle_launches[pusher][parity];
-    // host-side effects of the replayed steps: one sort, at the end
+    launches += ctx->cycle_launches[pusher][parity][fields];
+    // host-side effects of the replayed steps: one sort, at the end; L - 1 exchanges of the fields
+    if (merge && ((L - 1) & 1)) swap_fields(ctx);
     ctx->steps_done += L;
     ctx->q_prev_valid = false;
     std::swap(ctx->cell, ctx->cell_tmp);
@@ -1154,7 +1251,8 @@ extern "C" int fetdpic_step(fetdpic_ctx *ctx, long long nsteps, int pusher)
             CK(cudaStreamSynchronize(ctx->stream));
             collect_events(ctx);
         }
-        launches += enqueue_step(ctx, pusher, timed);
+        const bool merge = can_merge(ctx);
+        launches += enqueue_step(ctx, pusher, timed, merge && s > 0, merge && s + 1 < nsteps);
     }
     ctx->launches_acc += launches;
     CK(cudaGetLastError());
@@ -1634,9 +1732,9 @@ extern "C" int fetdpic_read_spai(fetdpic_ctx *ctx, int inst, long long *rowptr, 
 
 static void drop_graphs(fetdpic_ctx *ctx)
 {
-    for (auto &a : ctx->graph) for (auto &b : a) for (auto &c : b) for (auto &g : c)
+    for (auto &a : ctx->graph) for (auto &b : a) for (auto &c : b) for (auto &d : c) for (auto &g : d)
         if (g) { cudaGraphExecDestroy(g); g = nullptr; }
-    for (auto &a : ctx->cycle) for (auto &g : a)
+    for (auto &a : ctx->cycle) for (auto &b : a) for (auto &g : b)
         if (g) { cudaGraphExecDestroy(g); g = nullptr; }
 }
 
@@ -1722,7 +1820,8 @@ extern "C" int fetdpic_autotune(fetdpic_ctx *ctx, int pusher, int trial_steps, i
             const int n = si > 0 ? std::max(trial_steps, si) / si * si : trial_steps;
             enqueue_step(ctx, pusher, false);                           // warm-up
             CK(cudaEventRecord(t0, ctx->stream));
-            for (int k = 0; k < n; ++k) enqueue_step(ctx, pusher, false);
+            const bool merge = can_merge(ctx);
+            for (int k = 0; k < n; ++k) enqueue_step(ctx, pusher, false, merge && k > 0, merge && k + 1 < n);
             CK(cudaEventRecord(t1, ctx->stream));
             CK(cudaEventSynchronize(t1));
             float ms = 0.f;

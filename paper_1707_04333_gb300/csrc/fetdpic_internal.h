@@ -72,6 +72,37 @@ int build_spai(HostMesh &M, int level, std::string &msg);
 int electrostatic_solve(const HostMesh &M, const std::vector<double> &q, std::vector<double> &de,
                         int &iterations, double &rel_residual, std::string &msg);
 
+// The field update by patches (field_patches.cpp, kernels_field.cu).  A patch is
+// one thread block's share: triangles [t0, t0 + nt), the edges [e0, e0 + ne)
+// they touch first, and in xlist [x0, x0 + nx) the further edges whose curl its
+// rows need, those of its own triangles (the "ring", nring of them) first.
+// Inside the patch an edge is numbered by its place in that order.  Its rows of
+// the SPAI are its own free edges (nown) and the ring's (nringrow), each group
+// in slices of 32 of its own: row_loc [row0 + row] is a row's edge, soff
+// [slice0 + slice] where its pairs of entries start, col and val the entries
+// (pair by pair, 32 rows to a pair).
+struct FieldPatch { int t0, nt, e0, ne, x0, nx, nring, nown, nringrow, row0, slice0, pad; };
+static_assert(sizeof(FieldPatch) == 48, "FieldPatch layout");
+struct PatchSet {
+    bool ok = false;
+    int T = 0, max_r = 0, max_e = 0;        // largest ne + nx and ne + nring
+    std::vector<FieldPatch> patch;
+    std::vector<int> xlist;
+    std::vector<unsigned short> tloc;       // [F][4] local edges of each triangle
+    std::vector<unsigned short> row_loc, col;
+    std::vector<long long> soff;
+    std::vector<double> val;
+};
+// Stored triangles' edges (stored, global), row of each edge (-1: not free),
+// rows in CSR over stored global edges.
+struct PatchInput {
+    int F;
+    const int *tedge;
+    const int *row;
+    const long long *mrp; const int *mci; const double *mv;
+};
+PatchSet build_patches(const PatchInput &in, int T);
+
 // Same barycentric evaluation the kernels use (gradient form, no FMA).
 void host_lambdas(const HostMesh &M, int f, double x, double y, double *l);
 int host_locate(const HostMesh &M, double x, double y, int hint);
@@ -167,12 +198,13 @@ enum StatusBits : unsigned {
 // its memory is visible; it then lets the next kernel launch early in turn.
 // Without pdl this is a plain launch (and the wait returns at once).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_k(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args)
+inline cudaError_t launch_ks(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -180,6 +212,11 @@ inline cudaError_t launch_k(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k, args...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_k(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args)
+{
+    return launch_ks(pdl, k, grid, block, 0, st, args...);
 }
 
 __device__ __forceinline__ void pdl_begin()
@@ -227,15 +264,17 @@ struct StepArgs32 {
     unsigned spin;                          // polls of a bounded wait before it gives up (variant 5)
 };
 
+// The Faraday launches also clear the current accumulator (ifix, E edges) for
+// the particle kernel after them.
 void launch_faraday64(cudaStream_t st, int F, const Geo64 *geo, const Topo *topo, const double *e,
-                      double *b, Rec64 *rec);
+                      double *b, Rec64 *rec, int E, unsigned long long *ifix);
 // Applied fields folded into the FP32 field record (ext == NULL: none): per
 // instance (E_x, E_y, B_z, 0) times the amplitude (E) and the per-triangle
 // weights extw (NULL = 1); finst = instance of each triangle.
 struct __align__(16) ExtField { double ex, ey, bz, pad; };
 struct Ext32 { const int *finst; const ExtField *ext; const double *amp; const double2 *extw; double half_over_c; };
 void launch_faraday32(cudaStream_t st, int F, const CstA *csta, const CstB *cstb, const double2 *dtinv, const double *e,
-                      double *b, Rec32 *rec, float inv2c2, const Ext32 &x, bool pdl);
+                      double *b, Rec32 *rec, float inv2c2, const Ext32 &x, int E, unsigned long long *ifix, bool pdl);
 void launch_particles64(cudaStream_t st, int pusher, const StepArgs64 &a);
 void launch_particles32(cudaStream_t st, int pusher, const StepArgs32 &a);
 
@@ -264,6 +303,34 @@ struct AmpereArgs {
     unsigned *status;
 };
 void launch_ampere(cudaStream_t st, const AmpereArgs &a);
+
+// Ampere update by patches (one launch); with `faraday` the next step's Faraday
+// update and field record follow in the same launch: e, b and the current
+// accumulator then go from one buffer to the other (e_next, b_next; ifix_next
+// is cleared), because other patches still read the old values.
+struct FieldArgs {
+    int npatch; const FieldPatch *patch; const int *xlist; const ushort4 *tloc;
+    const unsigned short *row_loc; const unsigned *col; const long long *soff; const float *v32; const double *v64;
+    const int2 *efac; const double2 *ecoef; const int *einst; const double *inst_unit, *inst_dt;
+    const double *b; const unsigned long long *ifix; double *j, *d;
+    const double *e; double *e_next;
+    bool one_inst;                          // a single instance: no per-edge look-up
+    bool early;                             // b is complete before the previous kernel ends (read it before the wait)
+    bool pdl;
+    int max_r, max_e, T;
+    bool faraday;
+    double *b_next; unsigned long long *ifix_next;
+    const CstA *csta; const CstB *cstb; const double2 *dtinv; Rec32 *rec32; float inv2c2; Ext32 ext;   // FP32
+    const Geo64 *geo; const Topo *topo; Rec64 *rec64;                                                // FP64
+};
+// Triangles of a patch on a mesh of F triangles.
+int field_patch_size(int F, int sms);
+// Shared memory of one block; a context whose patches need more uses launch_ampere.
+size_t field_smem(bool f32, int max_r, int max_e);
+constexpr size_t FIELD_SMEM_MAX = 100 * 1024;
+// Prepares the kernels for `smem` bytes of shared memory (once per context).
+cudaError_t field_setup(size_t smem);
+void launch_field(cudaStream_t st, const FieldArgs &a);
 
 // Counting sort of particles by triangle, per species range.
 struct SortArgs {

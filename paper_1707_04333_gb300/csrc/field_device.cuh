@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "fetdpic_internal.h"
+#include "fp64_int.h"
 
 namespace fetdpic {
 
@@ -32,6 +33,18 @@ template <> __device__ __forceinline__ float ld_keep<float>(const float *p, unsi
     asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
     return v;
 }
+template <> __device__ __forceinline__ unsigned ld_keep<unsigned>(const unsigned *p, unsigned long long pol)
+{
+    unsigned v;
+    asm("ld.global.nc.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    return v;
+}
+template <> __device__ __forceinline__ float2 ld_keep<float2>(const float2 *p, unsigned long long pol)
+{
+    float2 v;
+    asm("ld.global.nc.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(p), "l"(pol));
+    return v;
+}
 template <> __device__ __forceinline__ double ld_keep<double>(const double *p, unsigned long long pol)
 {
     double v;
@@ -51,10 +64,51 @@ template <> __device__ __forceinline__ double2 ld_keep<double2>(const double2 *p
     return v;
 }
 
+// Faraday update of one triangle in FP64 and its FP32 field record: in a triangle
+// E(lambda) = sum_m s_m e_m (l_a grad l_b - l_b grad l_a) = sum_n l_n V_n with
+// V_n = s_{n-1} e_{n-1} grad l_{n+1} - s_{n+1} e_{n+1} grad l_{n-1}.  Stored
+// as dt/(2c) V_n = (s_{n-1} e_{n-1} G_{n+1} - s_{n+1} e_{n+1} G_{n-1}) / (2c^2)
+// (G = c dt grad l), so that q/m times it is alpha E / c; B_z^n stored as
+// (dt/2) B_z = (dt/2) (b^{n+1/2} + b^{n-1/2}) / (2A).  se = s_m e_m, bo =
+// b^{n-1/2}, di = (dt, 1/(2A)), (c0, c1) = CstA; returns b^{n+1/2}.
+__device__ __forceinline__ double faraday32_rec(int f, const double *se, double bo, double2 di, float4 c0, float4 c1,
+                                                int ew0, Rec32 *rec, float inv2c2, const Ext32 &x, bool ext)
+{
+    // G_2 = -(G_0 + G_1): the barycentric gradients of a triangle sum to zero
+    const float G[6] = {c0.x, c0.y, c0.z, c0.w, -(c0.x + c0.z), -(c0.y + c0.w)};
+    const double bn = bo - di.x * ((se[0] + se[1]) + se[2]);
+    float s[3] = {to_f32(se[0]) * inv2c2, to_f32(se[1]) * inv2c2, to_f32(se[2]) * inv2c2};
+    Rec32 r;
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+        const int nm = (n + 2) % 3, np = (n + 1) % 3;
+        r.v[2 * n] = s[nm] * G[2 * np] - s[np] * G[2 * nm];
+        r.v[2 * n + 1] = s[nm] * G[2 * np + 1] - s[np] * G[2 * nm + 1];
+    }
+    double bfield = (bn + bo) * di.y;
+    if (ext) {
+        // a uniform applied E adds the same value to every node coefficient (sum of lambdas = 1)
+        const int k = x.finst[f];
+        const ExtField X = x.ext[k];
+        double we = 1.0, wb = 1.0;
+        if (x.extw) { const double2 wv = x.extw[f]; we = wv.x; wb = wv.y; }
+        const double sa = x.amp[k] * we * di.x * x.half_over_c;
+        const float ax = (float)(sa * X.ex), ay = (float)(sa * X.ey);
+#pragma unroll
+        for (int n = 0; n < 3; ++n) { r.v[2 * n] += ax; r.v[2 * n + 1] += ay; }
+        bfield += wb * X.bz;                         // B_z = (b^{n+1/2} + b^{n-1/2}) / (2A) + B_ext
+    }
+    r.bz = to_f32(scale_i<-1>(di.x) * bfield);       // (dt / 2) B_z
+    float4 *rp = reinterpret_cast<float4 *>(rec + f);
+    rp[0] = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+    rp[1] = make_float4(r.v[4], r.v[5], r.bz, __int_as_float(ew0));
+    return bn;
+}
+
 // r = C^T [*mu^-1] b^{n+1/2} - i^{n+1/2} on edge e (Eq. (semi.dis.curl.2)),
 // with [*mu^-1] = 1/(mu0 A_f) folded into ecoef = s_f/(mu0 A_f).  The
 // fixed-point current is converted (unit = (q_ref/dt) 2^-shift per
-// instance), kept in j for reading, and cleared for the next step.  The dual
+// instance) and kept in j for reading.  The dual
 // flux d += dt r accumulates for the Gauss-law check (d == NULL: checks off);
 // r (FP64) is stored for the FP64 SpMV, r32 for the FP32 one (either NULL).
 __device__ __forceinline__ void curl_h_edge(const AmpereArgs &a, int e, unsigned long long keep)
@@ -65,7 +119,6 @@ __device__ __forceinline__ void curl_h_edge(const AmpereArgs &a, int e, unsigned
     if (fa.y >= 0) h += a.b[fa.y] * cf.y;
     const int in = ld_keep(a.einst + e, keep);
     const long long iv = (long long)a.ifix[e];
-    a.ifix[e] = 0ull;
     const double cur = (double)iv * a.inst_unit[in];
     const double rv = h - cur;
     if (a.r) a.r[e] = rv;

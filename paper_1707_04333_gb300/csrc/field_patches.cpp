@@ -1,0 +1,146 @@
+// Partition of the field update into patches of consecutive stored triangles
+// (a compact piece of the Hilbert curve), one thread block each
+// (kernels_field.cu): the edges a patch owns, the further edges whose curl it
+// recomputes, and its rows of the sparse approximate inverse with columns
+// numbered inside the patch.
+#include <algorithm>
+#include <thread>
+#include <vector>
+
+#include "fetdpic_internal.h"
+
+namespace fetdpic {
+
+namespace {
+
+// Patches [p0, p1) into S, offsets relative to S.
+void build_range(PatchSet &S, const PatchInput &in, const std::vector<int> &own, int T, int p0, int p1)
+{
+    std::vector<int> ring, ext, other, edge;
+    for (int p = p0; p < p1; ++p) {
+        FieldPatch P{};
+        P.t0 = p * T;
+        P.nt = std::min(T, in.F - P.t0);
+        P.e0 = own[p];
+        P.ne = own[p + 1] - own[p];
+        const int e1 = P.e0 + P.ne;
+        // edges of the patch's triangles that an earlier patch owns
+        ring.clear();
+        for (int k = 3 * P.t0; k < 3 * (P.t0 + P.nt); ++k) {
+            const int e = in.tedge[k];
+            if (e < P.e0 || e >= e1) ring.push_back(e);
+        }
+        std::sort(ring.begin(), ring.end());
+        ring.erase(std::unique(ring.begin(), ring.end()), ring.end());
+        P.nring = (int)ring.size();
+        // its rows (free edges: owned, then ring), and the other edges their columns name
+        edge.clear();
+        for (int e = P.e0; e < e1; ++e) if (in.row[e] >= 0) edge.push_back(e);
+        P.nown = (int)edge.size();
+        for (int e : ring) if (in.row[e] >= 0) edge.push_back(e);
+        P.nringrow = (int)edge.size() - P.nown;
+        ext.clear();
+        for (int e : edge)
+            for (long long q = in.mrp[in.row[e]]; q < in.mrp[in.row[e] + 1]; ++q)
+                if (in.mci[q] < P.e0 || in.mci[q] >= e1) ext.push_back(in.mci[q]);
+        std::sort(ext.begin(), ext.end());
+        ext.erase(std::unique(ext.begin(), ext.end()), ext.end());
+        other.clear();
+        std::set_difference(ext.begin(), ext.end(), ring.begin(), ring.end(), std::back_inserter(other));
+        P.x0 = (int)S.xlist.size();
+        P.nx = P.nring + (int)other.size();
+        S.xlist.insert(S.xlist.end(), ring.begin(), ring.end());
+        S.xlist.insert(S.xlist.end(), other.begin(), other.end());
+        auto local = [&](int e) {
+            if (e >= P.e0 && e < e1) return e - P.e0;
+            auto it = std::lower_bound(ring.begin(), ring.end(), e);
+            if (it != ring.end() && *it == e) return P.ne + (int)(it - ring.begin());
+            return P.ne + P.nring + (int)(std::lower_bound(other.begin(), other.end(), e) - other.begin());
+        };
+        S.max_r = std::max(S.max_r, P.ne + P.nx);
+        S.max_e = std::max(S.max_e, P.ne + P.nring);
+        for (int f = P.t0; f < P.t0 + P.nt; ++f)
+            for (int m = 0; m < 4; ++m) S.tloc.push_back(m < 3 ? (unsigned short)local(in.tedge[3 * f + m]) : 0);
+        // rows in slices of 32, pairs of entries column-major; owned rows and ring rows in slices of their own
+        P.row0 = (int)S.row_loc.size();
+        P.slice0 = (int)S.soff.size() - 1;
+        for (int part = 0; part < 2; ++part) {
+            const int r0 = part ? P.nown : 0, r1 = part ? P.nown + P.nringrow : P.nown;
+            for (int s0 = r0; s0 < r1; s0 += 32) {
+                long long w = 0;
+                for (int r = s0; r < std::min(r1, s0 + 32); ++r)
+                    w = std::max(w, in.mrp[in.row[edge[r]] + 1] - in.mrp[in.row[edge[r]]]);
+                w += w & 1;                 // entries in pairs; the added ones are 0
+                const size_t base = S.col.size();
+                S.col.resize(base + 32 * w, 0);
+                S.val.resize(base + 32 * w, 0.0);
+                for (int l = 0; l < 32; ++l) {
+                    const int r = s0 + l;
+                    S.row_loc.push_back(r < r1 ? (unsigned short)local(edge[r]) : 0);
+                    if (r >= r1) continue;
+                    const long long q0 = in.mrp[in.row[edge[r]]], n = in.mrp[in.row[edge[r]] + 1] - q0;
+                    // (padding names the row's own edge: 0 times another's NaN is not 0)
+                    for (long long k = n; k < w; ++k)
+                        S.col[base + 64 * (k / 2) + 2 * l + (k & 1)] = S.row_loc.back();
+                    for (long long k = 0; k < n; ++k) {
+                        const size_t q = base + 64 * (k / 2) + 2 * l + (k & 1);
+                        S.col[q] = (unsigned short)local(in.mci[q0 + k]);
+                        S.val[q] = in.mv[q0 + k];
+                    }
+                }
+                S.soff.push_back((long long)S.col.size() / 2);          // in pairs
+            }
+        }
+        S.patch.push_back(P);
+    }
+}
+
+}  // namespace
+
+PatchSet build_patches(const PatchInput &in, int T)
+{
+    const int np = in.F > 0 ? (in.F + T - 1) / T : 0;
+    // first edge of each patch: edges are numbered in the order the triangles touch them
+    std::vector<int> own(np + 1, 0);
+    int seen = 0;
+    for (int f = 0; f < in.F; ++f) {
+        if (f % T == 0) own[f / T] = seen;
+        for (int m = 0; m < 3; ++m) seen = std::max(seen, in.tedge[3 * f + m] + 1);
+    }
+    own[np] = seen;
+    const int nth = (int)std::max(1u, std::min({16u, std::thread::hardware_concurrency(), (unsigned)((np + 15) / 16)}));
+    std::vector<PatchSet> part(nth);
+    {
+        std::vector<std::thread> th;
+        for (int t = 0; t < nth; ++t)
+            th.emplace_back([&, t] {
+                part[t].soff.assign(1, 0);
+                build_range(part[t], in, own, T, (int)((long long)np * t / nth), (int)((long long)np * (t + 1) / nth));
+            });
+        for (auto &t : th) t.join();
+    }
+    PatchSet S;
+    S.soff.assign(1, 0);
+    S.T = T;
+    for (PatchSet &Q : part) {
+        const int x = (int)S.xlist.size(), r = (int)S.row_loc.size(), s = (int)S.soff.size() - 1;
+        const long long o = (long long)S.col.size() / 2;
+        for (FieldPatch P : Q.patch) {
+            P.x0 += x; P.row0 += r; P.slice0 += s;
+            S.patch.push_back(P);
+        }
+        S.xlist.insert(S.xlist.end(), Q.xlist.begin(), Q.xlist.end());
+        S.tloc.insert(S.tloc.end(), Q.tloc.begin(), Q.tloc.end());
+        S.row_loc.insert(S.row_loc.end(), Q.row_loc.begin(), Q.row_loc.end());
+        for (size_t k = 1; k < Q.soff.size(); ++k) S.soff.push_back(o + Q.soff[k]);
+        S.col.insert(S.col.end(), Q.col.begin(), Q.col.end());
+        S.val.insert(S.val.end(), Q.val.begin(), Q.val.end());
+        S.max_r = std::max(S.max_r, Q.max_r);
+        S.max_e = std::max(S.max_e, Q.max_e);
+        Q = PatchSet();
+    }
+    S.ok = np > 0 && S.max_r <= 65535;
+    return S;
+}
+
+}  // namespace fetdpic

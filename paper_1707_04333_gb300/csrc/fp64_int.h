@@ -213,4 +213,23 @@ F64I_FN long long rint_i(double a)
     return (h >> 31) ? -(long long)m : (long long)m;
 }
 
+// (float)a, nearest even, and (double)a, without the FP64 pipe (which does conversions too):
+// normal results; others through the hardware's conversion.
+F64I_FN float to_f32(double a)
+{
+    const u32 h = f64_hi(a), l = f64_lo(a);
+    const u32 u = (h & 0x7fffffffu) - (896u << 20);                    // exponent field of the result
+    if (u - 0x100000u >= (253u << 20)) return (float)a;
+    const u32 b = shl_pair(u, l, 3);
+    u32 o, carry;
+    add_round(l << 3, 0x7fffffffu + (b & 1u), 0u, 0u, b, carry, o);
+    return as_f32(o | (h & 0x80000000u));
+}
+F64I_FN double to_f64(float a)
+{
+    const u32 b = as_u32(a), m = b & 0x7fffffffu;
+    if (m - 0x800000u >= 0x7f000000u) return (double)a;
+    return f64_make(((m >> 3) + (896u << 20)) | (b & 0x80000000u), b << 29);
+}
+
 }  // namespace fetdpic

@@ -17,24 +17,30 @@
 
 namespace fetdpic {
 
-// Faraday update in FP64 (in place) and the FP32 field record: in a triangle
-// E(lambda) = sum_m s_m e_m (l_a grad l_b - l_b grad l_a) = sum_n l_n V_n with
-// V_n = s_{n-1} e_{n-1} grad l_{n+1} - s_{n+1} e_{n+1} grad l_{n-1}.  Stored
-// as dt/(2c) V_n = (s_{n-1} e_{n-1} G_{n+1} - s_{n+1} e_{n+1} G_{n-1}) / (2c^2)
-// (G = c dt grad l), so that q/m times it is alpha E / c; B_z^n stored as
-// (dt/2) B_z = (dt/2) (b^{n+1/2} + b^{n-1/2}) / (2A).
-__device__ __forceinline__ void faraday32_tri(int f, const CstA *__restrict__ csta, const CstB *__restrict__ cstb,
-                                              const double2 *__restrict__ dtinv, const double *e, double *b,
-                                              Rec32 *rec, float inv2c2, const Ext32 &x, bool ext)
+// Faraday update in FP64 (in place), the FP32 field record, and the current
+// accumulator cleared for the particle kernel that follows.
+template <bool EXT>
+__global__ void __launch_bounds__(256) k_faraday32(int F, const CstA *__restrict__ csta,
+                                                   const CstB *__restrict__ cstb,
+                                                   const double2 *__restrict__ dtinv,
+                                                   const double *__restrict__ e, double *__restrict__ b,
+                                                   Rec32 *__restrict__ rec, float inv2c2, Ext32 x, int E,
+                                                   unsigned long long *__restrict__ ifix)
 {
-    // the triangle's constants are static: loaded before the wait for the kernel that writes e
-    const float4 *cp = reinterpret_cast<const float4 *>(csta + f);
-    const float4 c0 = __ldg(cp), c1 = __ldg(cp + 1);
-    const CstB cb = cstb[f];
-    const double2 di = dtinv[f];                    // (dt, 1/(2A))
+    const int f = blockIdx.x * blockDim.x + threadIdx.x;
+    float4 c0, c1;
+    CstB cb{};
+    double2 di{};
+    if (f < F) {
+        // the triangle's constants are static: loaded before the wait for the kernel that writes e
+        const float4 *cp = reinterpret_cast<const float4 *>(csta + f);
+        c0 = __ldg(cp); c1 = __ldg(cp + 1);
+        cb = cstb[f];
+        di = dtinv[f];                                  // (dt, 1/(2A))
+    }
     pdl_begin();
-    // G_2 = -(G_0 + G_1): the barycentric gradients of a triangle sum to zero
-    const float G[6] = {c0.x, c0.y, c0.z, c0.w, -(c0.x + c0.z), -(c0.y + c0.w)};
+    for (int k = f; k < E; k += gridDim.x * blockDim.x) ifix[k] = 0ull;
+    if (f >= F) return;
     const int ew[3] = {cb.ew0, __float_as_int(c1.x), __float_as_int(c1.y)};
     double se[3];
 #pragma unroll
@@ -42,55 +48,17 @@ __device__ __forceinline__ void faraday32_tri(int f, const CstA *__restrict__ cs
         const double v = e[ew[m] >> 1];
         se[m] = (ew[m] & 1) ? -v : v;
     }
-    const double bo = b[f];
-    const double bn = bo - di.x * ((se[0] + se[1]) + se[2]);
-    b[f] = bn;
-    float s[3] = {(float)se[0] * inv2c2, (float)se[1] * inv2c2, (float)se[2] * inv2c2};
-    Rec32 r;
-#pragma unroll
-    for (int n = 0; n < 3; ++n) {
-        const int nm = (n + 2) % 3, np = (n + 1) % 3;
-        r.v[2 * n] = s[nm] * G[2 * np] - s[np] * G[2 * nm];
-        r.v[2 * n + 1] = s[nm] * G[2 * np + 1] - s[np] * G[2 * nm + 1];
-    }
-    double bfield = (bn + bo) * di.y;
-    if (ext) {
-        // a uniform applied E adds the same value to every node coefficient (sum of lambdas = 1)
-        const int k = x.finst[f];
-        const ExtField X = x.ext[k];
-        double we = 1.0, wb = 1.0;
-        if (x.extw) { const double2 wv = x.extw[f]; we = wv.x; wb = wv.y; }
-        const double sa = x.amp[k] * we * di.x * x.half_over_c;
-        const float ax = (float)(sa * X.ex), ay = (float)(sa * X.ey);
-#pragma unroll
-        for (int n = 0; n < 3; ++n) { r.v[2 * n] += ax; r.v[2 * n + 1] += ay; }
-        bfield += wb * X.bz;                         // B_z = (b^{n+1/2} + b^{n-1/2}) / (2A) + B_ext
-    }
-    r.bz = (float)(0.5 * di.x * bfield);
-    float4 *rp = reinterpret_cast<float4 *>(rec + f);
-    rp[0] = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
-    rp[1] = make_float4(r.v[4], r.v[5], r.bz, __int_as_float(ew[0]));
-}
-
-template <bool EXT>
-__global__ void __launch_bounds__(256) k_faraday32(int F, const CstA *__restrict__ csta,
-                                                   const CstB *__restrict__ cstb,
-                                                   const double2 *__restrict__ dtinv,
-                                                   const double *__restrict__ e, double *__restrict__ b,
-                                                   Rec32 *__restrict__ rec, float inv2c2, Ext32 x)
-{
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= F) { pdl_begin(); return; }
-    faraday32_tri(f, csta, cstb, dtinv, e, b, rec, inv2c2, x, EXT);
+    b[f] = faraday32_rec(f, se, b[f], di, c0, c1, cb.ew0, rec, inv2c2, x, EXT);
 }
 
 void launch_faraday32(cudaStream_t st, int F, const CstA *csta, const CstB *cstb, const double2 *dtinv,
-                      const double *e, double *b, Rec32 *rec, float inv2c2, const Ext32 &x, bool pdl)
+                      const double *e, double *b, Rec32 *rec, float inv2c2, const Ext32 &x, int E,
+                      unsigned long long *ifix, bool pdl)
 {
     if (F <= 0) return;
     const dim3 g((F + 255) / 256);
-    if (x.ext) launch_k(pdl, k_faraday32<true>, g, dim3(256), st, F, csta, cstb, dtinv, e, b, rec, inv2c2, x);
-    else launch_k(pdl, k_faraday32<false>, g, dim3(256), st, F, csta, cstb, dtinv, e, b, rec, inv2c2, x);
+    if (x.ext) launch_k(pdl, k_faraday32<true>, g, dim3(256), st, F, csta, cstb, dtinv, e, b, rec, inv2c2, x, E, ifix);
+    else launch_k(pdl, k_faraday32<false>, g, dim3(256), st, F, csta, cstb, dtinv, e, b, rec, inv2c2, x, E, ifix);
 }
 
 // --------------------------------------------------------------- pushers

@@ -17,9 +17,11 @@ namespace fetdpic {
 // fused with the per-triangle field record the particles gather from:
 // (s_m e_m) for the three local edges and B_z^n = (b^{n+1/2}+b^{n-1/2})/(2A).
 __global__ void k_faraday64(int F, const Geo64 *__restrict__ geo, const Topo *__restrict__ topo,
-                            const double *__restrict__ e, double *__restrict__ b, Rec64 *__restrict__ rec)
+                            const double *__restrict__ e, double *__restrict__ b, Rec64 *__restrict__ rec, int E,
+                            unsigned long long *__restrict__ ifix)
 {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int k = f; k < E; k += gridDim.x * blockDim.x) ifix[k] = 0ull;      // for the particle kernel
     if (f >= F) return;
     const Topo t = topo[f];
     double se[3];
@@ -43,10 +45,10 @@ __global__ void k_faraday64(int F, const Geo64 *__restrict__ geo, const Topo *__
 }
 
 void launch_faraday64(cudaStream_t st, int F, const Geo64 *geo, const Topo *topo, const double *e,
-                      double *b, Rec64 *rec)
+                      double *b, Rec64 *rec, int E, unsigned long long *ifix)
 {
     if (F <= 0) return;
-    k_faraday64<<<(F + 255) / 256, 256, 0, st>>>(F, geo, topo, e, b, rec);
+    k_faraday64<<<(F + 255) / 256, 256, 0, st>>>(F, geo, topo, e, b, rec, E, ifix);
 }
 
 // ------------------------------------------------------------ arithmetic

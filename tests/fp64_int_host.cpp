@@ -51,7 +51,7 @@ int main(int argc, char **argv)
 {
     const long long n = argc > 1 ? atoll(argv[1]) : 1000000;
     ulps = argc > 2 ? atoi(argv[2]) : 2;
-    long long bm = 0, bd = 0, bs = 0, br = 0;
+    long long bm = 0, bd = 0, bs = 0, br = 0, bc = 0;
     for (long long k = 0; k < n; ++k) {
         double a = value(k & 1 ? 2 : 400), b = value(k & 2 ? 2 : 400);
         if (k % 13 == 0) b = a * (1.0 + 0x1p-52 * (double)(rnd() % 3));      // quotients next to 1
@@ -61,11 +61,15 @@ int main(int argc, char **argv)
         bd += !same(div_i(a, b), a / b);
         if (a != 0.0) bs += !same(sqrt_i(std::fabs(a)), std::sqrt(std::fabs(a)));
         bm += !same(scale_i<2>(b), 4.0 * b) + !same(scale_i<-1>(a), 0.5 * a) + (is_neg(a) != (a < 0.0));
+        const double w = k % 23 == 0 ? a * 0.0 : value(k & 4 ? 2 : 160);
+        const float f = (float)w, g = as_f32((u32)rnd());
+        bc += as_u32(to_f32(w)) != as_u32(f) || !same(to_f64(f), (double)f);
+        if (g == g) bc += !same(to_f64(g), (double)g);
         double c = value(61);
         if (k % 7 == 0) c = (double)((long long)(rnd() % 4000000) - 2000000) * 0.5;
         br += rint_i(c) != (long long)std::nearbyint(c);
         if (k % 1000 == 0) br += rint_i(0x1p63) != 0x7fffffffffffffffll || rint_i(-0x1p70) != -0x7fffffffffffffffll - 1 || rint_i(0.0) != 0;
     }
-    printf("mul %lld div %lld sqrt %lld rint %lld\n", bm, bd, bs, br);
-    return (bm | bd | bs | br) != 0;
+    printf("mul %lld div %lld sqrt %lld rint %lld convert %lld\n", bm, bd, bs, br, bc);
+    return (bm | bd | bs | br | bc) != 0;
 }
