@@ -88,7 +88,6 @@ struct fetdpic_ctx {
     int block = 256;
     int *cell = nullptr, *cell_tmp = nullptr, *id = nullptr, *id_tmp = nullptr;
     void *f[4] = {nullptr, nullptr, nullptr, nullptr}, *f_tmp[4] = {nullptr, nullptr, nullptr, nullptr};
-    short *blk_sp = nullptr;
     short *chunk_sp = nullptr;               // species of each 32-particle chunk
     signed char *tshift = nullptr;           // periodic shift codes (FP64 walk), NULL without periodic walls
     double2 *period = nullptr;               // per instance
@@ -690,8 +689,8 @@ extern "C" int fetdpic_load_particles(fetdpic_ctx *ctx, int inst, double q, doub
 // Charge of the current particle state into q (fixed point).
 static void charge_now(fetdpic_ctx *ctx, unsigned long long *q)
 {
-    launch_charge(ctx->stream, ctx->p.precision == FETDPIC_FP32, ctx->P, ctx->cell, ctx->blk_sp, ctx->block,
-                  ctx->sp_dev, ctx->geo64, ctx->topo, ctx->f[0], ctx->f[1], q, ctx->N);
+    launch_charge(ctx->stream, ctx->p.precision == FETDPIC_FP32, ctx->P, ctx->cell, ctx->chunk_sp, ctx->sp_dev,
+                  ctx->geo64, ctx->topo, ctx->f[0], ctx->f[1], q, ctx->N);
 }
 
 // The Gauss-law check compares S~ d - q with its value at this point (after
@@ -825,7 +824,6 @@ static int finalize(fetdpic_ctx *ctx)
             ctx->f[k] = ctx->alloc<char>(fb * ctx->P);
             ctx->f_tmp[k] = ctx->alloc<char>(fb * ctx->P);
         }
-        ctx->blk_sp = ctx->alloc<short>(std::max<long long>(ctx->nblocks, 1));
         ctx->chunk_sp = ctx->alloc<short>(std::max<long long>(ctx->P / 32, 1));
         ctx->hist = ctx->alloc<int>(std::max<long long>(hist_n, 1));
         ctx->hoff = ctx->alloc<int>(std::max(ns, 1));
@@ -841,13 +839,11 @@ static int finalize(fetdpic_ctx *ctx)
     std::vector<int> cell(ctx->P, -1), id(ctx->P, -1);       // padding: no triangle, no load index
     std::vector<char> fh[4];
     for (int k = 0; k < 4; ++k) fh[k].assign(fb * ctx->P, 0);
-    std::vector<short> blk(ctx->nblocks);
     std::vector<short> chk(ctx->P / 32);
     for (int s = 0; s < ns; ++s) {
         const StagedSpecies &S = ctx->staged[s];
         const Species &D = ctx->sp[s];
         const HostMesh &M = ctx->mesh[S.inst];
-        for (long long b = D.off / ctx->block; b < (D.off + D.cap) / ctx->block; ++b) blk[b] = (short)s;
         for (long long b = D.off / 32; b < (D.off + D.cap) / 32; ++b) chk[b] = (short)s;
         // storage in stored-triangle order from the start (a counting sort; load order in id)
         std::vector<long long> start(M.nf + 1, 0), order(D.n);
@@ -881,7 +877,6 @@ static int finalize(fetdpic_ctx *ctx)
     rc = rc ? rc : upload(ctx, ctx->cell_tmp, cell.data(), cell.size());   // padding stays -1 in both buffers
     rc = rc ? rc : upload(ctx, ctx->id, id.data(), id.size());
     for (int k = 0; k < 4; ++k) rc = rc ? rc : upload(ctx, (char *)ctx->f[k], fh[k].data(), fh[k].size());
-    rc = rc ? rc : upload(ctx, ctx->blk_sp, blk.data(), blk.size());
     rc = rc ? rc : upload(ctx, ctx->chunk_sp, chk.data(), chk.size());
     rc = rc ? rc : upload(ctx, ctx->hoff, hoff.data(), hoff.size());
     rc = rc ? rc : upload(ctx, ctx->inst_unit, ctx->unit_host.data(), ctx->unit_host.size());
@@ -1017,12 +1012,17 @@ static void swap_fields(fetdpic_ctx *ctx)
     std::swap(ctx->ifix, ctx->ifix_alt);
 }
 
-// Whether the steps of one call may share a field update: Ampere's of one step
-// with Faraday's of the next (no stage events, whose stages are separate, and no
-// checks, which look at the current between them).
-static bool can_merge(const fetdpic_ctx *ctx)
+// Whether the step that `after` more steps follow may share its field update with
+// the next: Ampere's of one step with Faraday's of the next (not with stage events,
+// whose stages are separate; not the step of a check, which looks at the fields
+// between them).
+static bool checks_at(const fetdpic_ctx *ctx, long long step)
 {
-    return ctx->patches && ctx->p.time_stages == 0 && ctx->p.check_interval <= 0;
+    return ctx->p.check_interval > 0 && ctx->g0 && step % ctx->p.check_interval == 0;
+}
+static bool can_merge(const fetdpic_ctx *ctx, long long after)
+{
+    return after > 0 && ctx->patches && ctx->p.time_stages == 0 && !checks_at(ctx, ctx->steps_done + 1);
 }
 
 // One time step: Faraday (+ field record), particles, Ampere, periodic sort.
@@ -1032,8 +1032,7 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
 {
     long long launches = 0;
     const bool f32 = ctx->p.precision == FETDPIC_FP32;
-    const bool check = ctx->p.check_interval > 0 && ctx->g0 &&
-                       ((ctx->steps_done + 1) % ctx->p.check_interval == 0);
+    const bool check = checks_at(ctx, ctx->steps_done + 1);
     Ext32 x{};
     if (f32 && ctx->ext_on) {
         x.finst = ctx->face_inst; x.ext = ctx->ext_dev; x.amp = ctx->ext_amp; x.extw = ctx->extw;
@@ -1190,7 +1189,7 @@ static int cycle_step(fetdpic_ctx *ctx, int pusher, long long &launches)
     const int parity = ctx->cell == ctx->cell_a ? 0 : 1;
     const int L = ctx->p.sort_interval;
     const int fields = ctx->e == ctx->e_a ? 0 : 1;
-    const bool merge = can_merge(ctx);
+    const bool merge = can_merge(ctx, L - 1);
     cudaGraphExec_t &g = ctx->cycle[pusher][parity][fields];
     if (!g) {
         cudaGraph_t graph = nullptr;
@@ -1234,6 +1233,7 @@ extern "C" int fetdpic_step(fetdpic_ctx *ctx, long long nsteps, int pusher)
     long long launches = 0;
     const bool timed = ctx->p.time_stages != 0;
     const bool graphs = ctx->p.use_graphs != 0 && !timed && ctx->p.check_interval <= 0;
+    bool begun = false;                          // the previous step's field update carried this one's Faraday
     for (long long s = 0; s < nsteps; ++s) {
         if (graphs) {
             const int L = ctx->p.sort_interval;
@@ -1251,8 +1251,9 @@ extern "C" int fetdpic_step(fetdpic_ctx *ctx, long long nsteps, int pusher)
             CK(cudaStreamSynchronize(ctx->stream));
             collect_events(ctx);
         }
-        const bool merge = can_merge(ctx);
-        launches += enqueue_step(ctx, pusher, timed, merge && s > 0, merge && s + 1 < nsteps);
+        const bool more = can_merge(ctx, nsteps - 1 - s);
+        launches += enqueue_step(ctx, pusher, timed, begun, more);
+        begun = more;
     }
     ctx->launches_acc += launches;
     CK(cudaGetLastError());
@@ -1820,8 +1821,8 @@ extern "C" int fetdpic_autotune(fetdpic_ctx *ctx, int pusher, int trial_steps, i
             const int n = si > 0 ? std::max(trial_steps, si) / si * si : trial_steps;
             enqueue_step(ctx, pusher, false);                           // warm-up
             CK(cudaEventRecord(t0, ctx->stream));
-            const bool merge = can_merge(ctx);
-            for (int k = 0; k < n; ++k) enqueue_step(ctx, pusher, false, merge && k > 0, merge && k + 1 < n);
+            for (int k = 0; k < n; ++k)
+                enqueue_step(ctx, pusher, false, k > 0 && can_merge(ctx, 1), can_merge(ctx, n - 1 - k));
             CK(cudaEventRecord(t1, ctx->stream));
             CK(cudaEventSynchronize(t1));
             float ms = 0.f;

@@ -349,9 +349,8 @@ void launch_sort(cudaStream_t st, const SortArgs &a);
 
 
 // Conservation checks (kernels_check.cu).
-void launch_charge(cudaStream_t st, bool fp32, long long P, const int *cell, const short *blk_sp, int block,
-                   const Species *sp, const Geo64 *geo, const Topo *topo, const void *f0, const void *f1,
-                   unsigned long long *q, int N);
+void launch_charge(cudaStream_t st, bool fp32, long long P, const int *cell, const short *chunk_sp, const Species *sp,
+                   const Geo64 *geo, const Topo *topo, const void *f0, const void *f1, unsigned long long *q, int N);
 void launch_dce(cudaStream_t st, int N, const int *nrp, const int *nedge, const int *ninst,
                 const unsigned long long *ifix, const unsigned long long *q0, const unsigned long long *q1, double *out);
 // Field probe: E(x_p) = sum_m w_m e[eg_m], w_m = s_m (l_a grad l_b - l_b grad l_a)
