@@ -328,8 +328,8 @@ int fetdpic_check(fetdpic_ctx *ctx, int inst, double *dce_max, double *dgl_max, 
  * graphs.  EINVAL on a non-finite weight.
  *
  * fetdpic_set_external_amplitude: a for the steps enqueued after this call
- * (stream-ordered; steps replayed from graphs see it too).  Returns once the
- * value is on the device.  EINVAL on a non-finite a. */
+ * (stream-ordered; steps replayed from graphs see it too); does not wait.
+ * EINVAL on a non-finite a. */
 int fetdpic_set_external_profile(fetdpic_ctx *ctx, int inst, const double *w);
 int fetdpic_set_external_amplitude(fetdpic_ctx *ctx, int inst, double amplitude);
 

@@ -123,6 +123,9 @@ struct fetdpic_ctx {
     std::vector<std::vector<char>> abs_nodes; // per instance: nodes off the PEC walls (absolute reference 0)
     // reusable device scratch for host <-> device transfers of particle state
     void *xfer = nullptr; size_t xfer_bytes = 0;
+    // page-locked host memory: small reads come back in one copy each, with the status word behind
+    // them, and one wait (SMALL_READ bytes for them, then the status)
+    char *pin = nullptr;
     // asynchronous particle reads: staging of their own (one region per species), copied to the
     // host on the io stream while the context stream goes on; set up by the first such read
     cudaStream_t io = nullptr;
@@ -164,6 +167,7 @@ struct fetdpic_ctx {
             if (p.dev_free) p.dev_free(q, p.alloc_user);
             else cudaFree(q);
         }
+        if (pin) cudaFreeHost(pin);
         for (auto &x : ev) cudaEventDestroy(x);
         for (auto &x : ev_rd_done) if (x) cudaEventDestroy(x);
         if (ev_rd) cudaEventDestroy(ev_rd);
@@ -209,6 +213,10 @@ struct fetdpic_ctx {
     }
 };
 
+// Reads of up to this many bytes go through the context's page-locked buffer (one copy and one wait:
+// a particle read took three pageable copies, each a wait of its own, and a fourth for the status).
+constexpr size_t SMALL_READ = 256 * 1024;
+
 // FP32 particle-kernel variant when the caller names none (see fetdpic_params.kernel_variant)
 constexpr int FP32_DEFAULT_VARIANT = 22;
 
@@ -238,21 +246,22 @@ static int map_status(fetdpic_ctx *ctx, unsigned st)
     return FETDPIC_OK;
 }
 
-// Reads the device status word and clears it when set, so a latched fault is
-// reported once; returns the mapped status (the caller's stream must be idle).
+// Waits for the context stream with the device status word behind its work, and clears the word when
+// set, so a latched fault is reported once; returns the mapped status.
 static int take_status(fetdpic_ctx *ctx)
 {
-    if (!ctx->status) return FETDPIC_OK;
-    unsigned st = 0;
-    CK(cudaMemcpy(&st, ctx->status, sizeof(unsigned), cudaMemcpyDeviceToHost));
-    if (st) CK(cudaMemset(ctx->status, 0, sizeof(unsigned)));
+    unsigned *st = reinterpret_cast<unsigned *>(ctx->pin + SMALL_READ);
+    CK(cudaMemcpyAsync(st, ctx->status, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    const unsigned s = *st;
+    if (s) CK(cudaMemset(ctx->status, 0, sizeof(unsigned)));
     // a step that timed out is incomplete: drop the current it deposited, and the counts a grid
     // barrier that gave up left behind
-    if (st & ST_TIMEOUT) {
+    if (s & ST_TIMEOUT) {
         if (ctx->gbar) CK(cudaMemset(ctx->gbar, 0, sizeof(unsigned) * GBAR_WORDS));
         if (ctx->ifix) CK(cudaMemset(ctx->ifix, 0, sizeof(unsigned long long) * ctx->E));
     }
-    return map_status(ctx, st);
+    return map_status(ctx, s);
 }
 
 extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int n_inst, const fetdpic_instance *inst)
@@ -287,6 +296,12 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
     CK(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
+
+    if (cudaHostAlloc((void **)&ctx->pin, SMALL_READ + 256, cudaHostAllocDefault) != cudaSuccess) {
+        ctx->pin = nullptr;
+        cudaGetLastError();
+        return FETDPIC_ENOMEM;
+    }
 
     // ---- host setup per instance
     ctx->mesh.resize(n_inst);
@@ -1263,10 +1278,10 @@ extern "C" int fetdpic_step(fetdpic_ctx *ctx, long long nsteps, int pusher)
 extern "C" int fetdpic_sync(fetdpic_ctx *ctx)
 {
     if (!ctx) return FETDPIC_EINVAL;
-    CK(cudaStreamSynchronize(ctx->stream));
+    const int rc = take_status(ctx);                       // waits for the stream
     if (ctx->io) CK(cudaStreamSynchronize(ctx->io));      // host copies of asynchronous reads
     collect_events(ctx);
-    return take_status(ctx);
+    return rc;
 }
 
 // Reusable device scratch for particle-state transfers (grown on demand).
@@ -1429,15 +1444,35 @@ extern "C" int fetdpic_read(fetdpic_ctx *ctx, int inst, double *e, double *b, do
         if (b) launch_gather_field(ctx->stream, M.nf, co, ctx->tri_c2i, ctx->b, ob);
         if (j) launch_gather_field(ctx->stream, M.ne, eo, ctx->edge_c2i, ctx->j, oj);
         CK(cudaGetLastError());
-        if (e) CK(cudaMemcpyAsync(e, oe, sizeof(double) * M.ne, cudaMemcpyDeviceToHost, ctx->stream));
-        if (b) CK(cudaMemcpyAsync(b, ob, sizeof(double) * M.nf, cudaMemcpyDeviceToHost, ctx->stream));
-        if (j) CK(cudaMemcpyAsync(j, oj, sizeof(double) * M.ne, cudaMemcpyDeviceToHost, ctx->stream));
+        const size_t be = sizeof(double) * M.ne, bf = sizeof(double) * M.nf;
+        if ((e || b || j) && 2 * be + bf <= SMALL_READ) {
+            CK(cudaMemcpyAsync(ctx->pin, oe, 2 * be + bf, cudaMemcpyDeviceToHost, ctx->stream));
+            if (x || u || cell) {                    // the buffer is used again below
+                CK(cudaStreamSynchronize(ctx->stream));
+            } else {
+                const int rc = take_status(ctx);
+                if (rc == FETDPIC_ECUDA) return rc;
+                if (e) std::memcpy(e, ctx->pin, be);
+                if (j) std::memcpy(j, ctx->pin + be, be);
+                if (b) std::memcpy(b, ctx->pin + 2 * be, bf);
+                return rc;
+            }
+            if (e) std::memcpy(e, ctx->pin, be);
+            if (j) std::memcpy(j, ctx->pin + be, be);
+            if (b) std::memcpy(b, ctx->pin + 2 * be, bf);
+        } else {
+            if (e) CK(cudaMemcpyAsync(e, oe, be, cudaMemcpyDeviceToHost, ctx->stream));
+            if (b) CK(cudaMemcpyAsync(b, ob, bf, cudaMemcpyDeviceToHost, ctx->stream));
+            if (j) CK(cudaMemcpyAsync(j, oj, be, cudaMemcpyDeviceToHost, ctx->stream));
+        }
     }
-    CK(cudaStreamSynchronize(ctx->stream));
     if (x || u || cell) {
         int rc = finalize(ctx);
         if (rc) return rc;
-        if (species < 0 || species >= (int)ctx->sp.size()) return ctx->fail(FETDPIC_EINVAL, "bad species");
+        if (species < 0 || species >= (int)ctx->sp.size()) {
+            CK(cudaStreamSynchronize(ctx->stream));
+            return ctx->fail(FETDPIC_EINVAL, "bad species");
+        }
         const Species &D = ctx->sp[species];
         if (D.n > 0) {
             const size_t bx = sizeof(double) * 2 * D.n, bc = sizeof(int) * D.n;
@@ -1453,10 +1488,18 @@ extern "C" int fetdpic_read(fetdpic_ctx *ctx, int inst, double *e, double *b, do
                 launch_unsort64(ctx->stream, D.n, ctx->cell, ctx->id, (double *)ctx->f[0], (double *)ctx->f[1],
                                 (double *)ctx->f[2], (double *)ctx->f[3], D.off, D.cap, ctx->tri_i2c, ox, ou, oc);
             CK(cudaGetLastError());
+            if (2 * bx + bc <= SMALL_READ) {
+                CK(cudaMemcpyAsync(ctx->pin, st, 2 * bx + bc, cudaMemcpyDeviceToHost, ctx->stream));
+                const int rc = take_status(ctx);
+                if (rc == FETDPIC_ECUDA) return rc;
+                if (x) std::memcpy(x, ctx->pin, bx);
+                if (u) std::memcpy(u, ctx->pin + bx, bx);
+                if (cell) std::memcpy(cell, ctx->pin + 2 * bx, bc);
+                return rc;
+            }
             if (x) CK(cudaMemcpyAsync(x, ox, bx, cudaMemcpyDeviceToHost, ctx->stream));
             if (u) CK(cudaMemcpyAsync(u, ou, bx, cudaMemcpyDeviceToHost, ctx->stream));
             if (cell) CK(cudaMemcpyAsync(cell, oc, bc, cudaMemcpyDeviceToHost, ctx->stream));
-            CK(cudaStreamSynchronize(ctx->stream));
         }
     }
     return take_status(ctx);
@@ -1630,8 +1673,8 @@ extern "C" int fetdpic_set_external_amplitude(fetdpic_ctx *ctx, int inst, double
     if (!std::isfinite(amplitude)) return ctx->fail(FETDPIC_EINVAL, "non-finite amplitude");
     CK(cudaSetDevice(ctx->device));
     // stream-ordered: steps enqueued before see the old value, later ones the new
-    CK(cudaMemcpyAsync(ctx->ext_amp + inst, &amplitude, sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    launch_set_value(ctx->stream, ctx->ext_amp + inst, amplitude);
+    CK(cudaGetLastError());
     return FETDPIC_OK;
 }
 
@@ -1696,14 +1739,16 @@ extern "C" int fetdpic_read_probes(fetdpic_ctx *ctx, double *exy, long long max_
     CK(cudaMemcpy(&cnt, ctx->probe_count, sizeof(cnt), cudaMemcpyDeviceToHost));
     const long long have = std::min<long long>((long long)cnt, ctx->probe_cap);
     const long long take = std::min(have, max_rows);
+    // the last `take` rows, oldest first: one piece of the ring, or two where it wraps
     const size_t row_bytes = sizeof(double2) * (size_t)ctx->probe_n;
-    for (long long k = 0; k < take; ++k) {
-        // oldest of the last `take` rows first
-        const unsigned long long step = cnt - (unsigned long long)take + (unsigned long long)k;
-        const long long r = (long long)(step % (unsigned long long)ctx->probe_cap);
-        CK(cudaMemcpyAsync(exy + (size_t)k * 2 * (size_t)ctx->probe_n, ctx->probe_ring + (size_t)r * ctx->probe_n,
-                           row_bytes, cudaMemcpyDeviceToHost, ctx->stream));
-    }
+    const long long first = take > 0 ? (long long)((cnt - (unsigned long long)take) % (unsigned long long)ctx->probe_cap) : 0;
+    const long long run = std::min(take, ctx->probe_cap - first);
+    if (run > 0)
+        CK(cudaMemcpyAsync(exy, ctx->probe_ring + (size_t)first * ctx->probe_n, row_bytes * run, cudaMemcpyDeviceToHost,
+                           ctx->stream));
+    if (take > run)
+        CK(cudaMemcpyAsync(exy + (size_t)run * 2 * (size_t)ctx->probe_n, ctx->probe_ring, row_bytes * (take - run),
+                           cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     if (rows) *rows = take;
     if (total) *total = (long long)cnt;

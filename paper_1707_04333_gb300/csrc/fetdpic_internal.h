@@ -381,6 +381,9 @@ void launch_ingest(cudaStream_t st, long long n, long long cap, long long off, i
 // to the caller's instance-local index.  A slot with triangle -1 and a load
 // index in [0, n) is a particle dropped by a write: its entry gets NaN
 // position and momentum and triangle -1.
+// *dst = v, in stream order.
+void launch_set_value(cudaStream_t st, double *dst, double v);
+
 // dst[k] = src[off + c2i[off + k]]: one instance's edge or triangle values in the caller's order.
 void launch_gather_field(cudaStream_t st, int n, int off, const int *c2i, const double *src, double *dst);
 

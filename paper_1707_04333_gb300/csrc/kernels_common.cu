@@ -450,6 +450,9 @@ void launch_ingest(cudaStream_t st, long long n, long long cap, long long off, i
                                                             geo, inv_c, cell_o, id_o, f0, f1, f2, f3, status);
 }
 
+__global__ void k_set_value(double *dst, double v) { *dst = v; }
+void launch_set_value(cudaStream_t st, double *dst, double v) { k_set_value<<<1, 1, 0, st>>>(dst, v); }
+
 __global__ void __launch_bounds__(256) k_gather_field(int n, int off, const int *__restrict__ c2i,
                                                       const double *__restrict__ src, double *__restrict__ dst)
 {
