@@ -127,7 +127,8 @@ typedef struct {
                                 Hybrids: 17 = variant 12 for the first 6 steps after a sort and
                                 variant 14 after them, 18 = the same switching after 4 steps,
                                 21 = variant 19 for 6 steps then 14, 22 = variant 19 for 6
-                                steps then 20.  0 = default (22).  All give identical results.
+                                steps then 20.  0 = chosen from these by the number of particles,
+                                particles per triangle and pusher.  All give identical results.
                                 Other values: FETDPIC_EINVAL. */
     void *cuda_stream;       /* cudaStream_t to run on; NULL = a stream owned by the context */
     /* Optional device allocator (e.g. a framework's caching allocator).  NULL = cudaMalloc/cudaFree. */

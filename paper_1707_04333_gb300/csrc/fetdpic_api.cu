@@ -83,6 +83,7 @@ struct fetdpic_ctx {
     std::vector<Species> sp;
     Species *sp_dev = nullptr;
     Sp32 *sp32_dev = nullptr;
+    int sms = 0;                             // of the device
     bool soft64 = false;                     // FP64 constants within the integer arithmetic's range
     long long P = 0, nblocks = 0;
     int block = 256;
@@ -215,10 +216,7 @@ struct fetdpic_ctx {
 
 // Reads of up to this many bytes go through the context's page-locked buffer (one copy and one wait:
 // a particle read took three pageable copies, each a wait of its own, and a fourth for the status).
-constexpr size_t SMALL_READ = 256 * 1024;
-
-// FP32 particle-kernel variant when the caller names none (see fetdpic_params.kernel_variant)
-constexpr int FP32_DEFAULT_VARIANT = 22;
+constexpr size_t SMALL_READ = 64 * 1024;
 
 #define CK(call)                                                                     \
     do {                                                                             \
@@ -284,13 +282,10 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
     if (P.block_size < 32 || P.block_size > 256 || (P.block_size & 31) || (SPECIES_ALIGN % P.block_size))
         return FETDPIC_EINVAL;
     if (P.record_walk < 0) return FETDPIC_EINVAL;
-    // untuned FP32 default: the hybrid 22 (two particles per thread in 64-thread blocks, 28 warps
-    // per SM for 6 steps after a sort, then 24 warps per SM with a deposit window), measured fastest
-    // on the benchmark workload
     if (P.kernel_variant < 0 || P.kernel_variant == 1 || P.kernel_variant > 22) return FETDPIC_EINVAL;
-    if (P.kernel_variant == 0) P.kernel_variant = FP32_DEFAULT_VARIANT;
     ctx->block = P.block_size;
     CK(cudaGetDevice(&ctx->device));
+    CK(cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device));
     if (P.cuda_stream) ctx->stream = (cudaStream_t)P.cuda_stream;
     else { CK(cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking)); ctx->own_stream = true; }
     CK(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
@@ -435,10 +430,8 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         for (int f = 0; f < ctx->F; ++f)
             for (int m = 0; m < 3; ++m) te[3 * (size_t)f + m] = tp[f].ew[m] >> 1;
         for (size_t r = 0; r < mrow.size(); ++r) row[mrow[r]] = (int)r;
-        int sms = 0;
-        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
         ps = build_patches(PatchInput{ctx->F, te.data(), row.data(), mrp.data(), mci.data(), mv.data()},
-                           field_patch_size(ctx->F, sms));
+                           field_patch_size(ctx->F, ctx->sms));
         ctx->patches = ps.ok && field_smem(f32, ps.max_r, ps.max_e) <= FIELD_SMEM_MAX;
     }
     // else sliced ELL over all rows (32 rows per slice, column-major inside a slice)
@@ -464,6 +457,24 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
             }
             soff.push_back(base + 32 * wmax);
         }
+    }
+    // the patches' tables one after another, each on a 256-byte boundary
+    std::vector<char> tables;
+    std::vector<size_t> at;
+    if (ctx->patches) {
+        auto put = [&](const void *p, size_t bytes) {
+            at.push_back((tables.size() + 255) / 256 * 256);
+            tables.resize(at.back() + bytes);
+            std::memcpy(tables.data() + at.back(), p, bytes);
+        };
+        tables.reserve(ps.patch.size() * sizeof(FieldPatch) + 4 * ps.xlist.size() + 2 * ps.tloc.size() +
+                       2 * ps.row_loc.size() + 2 * ps.col.size() + 8 * ps.soff.size() + 6 * 256);
+        put(ps.patch.data(), ps.patch.size() * sizeof(FieldPatch));
+        put(ps.xlist.data(), ps.xlist.size() * sizeof(int));
+        put(ps.tloc.data(), ps.tloc.size() * sizeof(unsigned short));
+        put(ps.row_loc.data(), ps.row_loc.size() * sizeof(unsigned short));
+        put(ps.col.data(), ps.col.size() * sizeof(unsigned short));
+        put(ps.soff.data(), ps.soff.size() * sizeof(long long));
     }
     const std::vector<double> &mat = ctx->patches ? ps.val : sv;
     std::vector<float> sv32;
@@ -543,18 +554,20 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         else ctx->m_v = ctx->alloc<double>(mat.size());
         if (ctx->patches) {
             FieldArgs &A = ctx->field;
-            A.patch = ctx->alloc<FieldPatch>(ps.patch.size());
-            A.xlist = ctx->alloc<int>(ps.xlist.size());
-            A.tloc = ctx->alloc<ushort4>(ctx->F);
-            A.row_loc = ctx->alloc<unsigned short>(ps.row_loc.size());
-            A.col = ctx->alloc<unsigned>(ps.col.size() / 2);
-            A.soff = ctx->alloc<long long>(ps.soff.size());
-            ctx->e_alt = ctx->alloc<double>(ctx->E);
-            ctx->b_alt = ctx->alloc<double>(ctx->F);
-            ctx->ifix_alt = ctx->alloc<unsigned long long>(ctx->E);
-            CK(cudaMemset(ctx->e_alt, 0, sizeof(double) * ctx->E));  // PEC edges are 0 in both buffers
-            CK(cudaMemset(ctx->b_alt, 0, sizeof(double) * ctx->F));
-            CK(cudaMemset(ctx->ifix_alt, 0, sizeof(unsigned long long) * ctx->E));
+            // the tables in one piece, the second buffers in another (cleared: PEC edges are 0 in both)
+            char *tab = ctx->alloc<char>(tables.size());
+            A.patch = (const FieldPatch *)(tab + at[0]);
+            A.xlist = (const int *)(tab + at[1]);
+            A.tloc = (const ushort4 *)(tab + at[2]);
+            A.row_loc = (const unsigned short *)(tab + at[3]);
+            A.col = (const unsigned *)(tab + at[4]);
+            A.soff = (const long long *)(tab + at[5]);
+            const size_t be = ((size_t)ctx->E * 8 + 255) / 256 * 256, bf = ((size_t)ctx->F * 8 + 255) / 256 * 256;
+            char *alt = ctx->alloc<char>(2 * be + bf);
+            CK(cudaMemsetAsync(alt, 0, 2 * be + bf, ctx->stream));
+            ctx->e_alt = (double *)alt;
+            ctx->ifix_alt = (unsigned long long *)(alt + be);
+            ctx->b_alt = (double *)(alt + 2 * be);
             A.npatch = (int)ps.patch.size();
             A.max_r = ps.max_r; A.max_e = ps.max_e; A.T = ps.T;
             CK(field_setup(field_smem(f32, ps.max_r, ps.max_e)));
@@ -649,13 +662,7 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         rc = rc ? rc : upload(ctx, ctx->edge_c2i, ec2i.data(), ec2i.size());
     }
     if (ctx->patches) {
-        const FieldArgs &A = ctx->field;
-        rc = rc ? rc : upload(ctx, const_cast<FieldPatch *>(A.patch), ps.patch.data(), ps.patch.size());
-        rc = rc ? rc : upload(ctx, const_cast<int *>(A.xlist), ps.xlist.data(), ps.xlist.size());
-        rc = rc ? rc : upload(ctx, (unsigned short *)const_cast<ushort4 *>(A.tloc), ps.tloc.data(), ps.tloc.size());
-        rc = rc ? rc : upload(ctx, const_cast<unsigned short *>(A.row_loc), ps.row_loc.data(), ps.row_loc.size());
-        rc = rc ? rc : upload(ctx, (unsigned short *)const_cast<unsigned *>(A.col), ps.col.data(), ps.col.size());
-        rc = rc ? rc : upload(ctx, const_cast<long long *>(A.soff), ps.soff.data(), ps.soff.size());
+        rc = rc ? rc : upload(ctx, (char *)ctx->field.patch, tables.data(), tables.size());
     } else {
         rc = rc ? rc : upload(ctx, ctx->m_soff, soff.data(), soff.size());
         ctx->m_entries = soff.back();
@@ -940,29 +947,43 @@ static StepArgs64 args64(fetdpic_ctx *ctx)
 struct Hybrid { int v, early, late, steps; };
 static constexpr Hybrid HYBRIDS[] = {{17, 12, 14, 6}, {18, 12, 14, 4}, {21, 19, 14, 6}, {22, 19, 20, 6}};
 
-static const Hybrid *hybrid_of(int v)
-{
-    for (const Hybrid &h : HYBRIDS)
-        if (h.v == v) return &h;
-    return nullptr;
-}
-
-// FP32 particle-kernel variant of the coming step.
-static int step_variant(const fetdpic_ctx *ctx)
+// The FP32 kernels a context runs, by its variant; one kernel throughout where early and late agree.
+// Variant 0, nothing chosen by the caller (device us a step, a sort every 16 steps):
+//   - up to one 64-particle chunk per SM: the kernel with one particle per lane is through it soonest
+//     (64 particles: 6.15 against 6.7 with variant 22; 4,000: 7.0 against 7.6; with two chunks per
+//     SM variant 12 is ahead, 8.72 against 8.93);
+//   - fewer than twelve particles per triangle: runs are short from the start and the window's flush
+//     does not pay (two per triangle: 42.5 with variant 12, 44.7 with 22; eight: 18.7 against 20.1);
+//   - else an early and a late kernel.  Early, 28 warps per SM for the Vay pusher, 24 for the others,
+//     whose kernels spill at 72 registers (8 M particles, Higuera-Cary: 130.5 against 134.3).  Late, the 20-warp window kernel up to 2 M particles,
+//     where its few more particles per warp cost less than registers held back from it (1.1 M in 16
+//     instances: 53.8 against 55.6), the 24-warp one above (8 M: 130.2 against 131.3).
+static Hybrid kernels_of(const fetdpic_ctx *ctx, int pusher)
 {
     const int v = ctx->p.kernel_variant;
-    const Hybrid *h = hybrid_of(v);
-    if (!h) return v;
-    const long long since = ctx->p.sort_interval > 0 ? ctx->steps_done % ctx->p.sort_interval : ctx->steps_done;
-    return since < h->steps ? h->early : h->late;
+    for (const Hybrid &h : HYBRIDS)
+        if (h.v == v) return h;
+    if (v != 0) return Hybrid{v, v, v, 0};
+    const long long n64 = ctx->P / 64;
+    if (n64 <= ctx->sms) return Hybrid{0, 4, 4, 0};
+    if (ctx->P < 12ll * ctx->F) return Hybrid{0, 12, 12, 0};
+    return Hybrid{0, pusher == FETDPIC_VAY ? 19 : 12, n64 < 32768 ? 14 : 20, 6};
 }
 
-static StepArgs32 args32(fetdpic_ctx *ctx)
+// Whether the coming step runs the late kernel.
+static bool late_step(const fetdpic_ctx *ctx, const Hybrid &h)
+{
+    const long long since = ctx->p.sort_interval > 0 ? ctx->steps_done % ctx->p.sort_interval : ctx->steps_done;
+    return since >= h.steps;
+}
+
+static StepArgs32 args32(fetdpic_ctx *ctx, int pusher)
 {
     StepArgs32 a{};
+    const Hybrid h = kernels_of(ctx, pusher);
     a.csta = ctx->csta; a.cstb = ctx->cstb; a.rec = ctx->rec32;
     a.sp = ctx->sp32_dev; a.chunk_sp = ctx->chunk_sp; a.nchunks = ctx->P / 32;
-    a.variant = step_variant(ctx);
+    a.variant = late_step(ctx, h) ? h.late : h.early;
     a.l0 = (float *)ctx->f[0]; a.l1 = (float *)ctx->f[1]; a.ux = (float *)ctx->f[2]; a.uy = (float *)ctx->f[3];
     a.cell = ctx->cell;
     a.ifix = ctx->ifix; a.status = ctx->status;
@@ -1079,7 +1100,7 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
     if (check && !ctx->q_prev_valid) { charge_now(ctx, ctx->q0); launches += 2; }
     if (ctx->nblocks > 0) {
         if (f32) {
-            StepArgs32 a = args32(ctx);
+            StepArgs32 a = args32(ctx, pusher);
             a.pdl = !timed;
             launch_particles32(ctx->stream, pusher, a);
         }
@@ -1163,8 +1184,7 @@ static int graph_step(fetdpic_ctx *ctx, int pusher, long long &launches)
     const bool sorts = ctx->p.sort_interval > 0 && ctx->nblocks > 0 &&
                        (ctx->steps_done + 1) % ctx->p.sort_interval == 0;
     const int parity = ctx->cell == ctx->cell_a ? 0 : 1;
-    const Hybrid *hy = hybrid_of(ctx->p.kernel_variant);
-    const int late = ctx->p.precision == FETDPIC_FP32 && hy && step_variant(ctx) == hy->late ? 1 : 0;
+    const int late = ctx->p.precision == FETDPIC_FP32 && late_step(ctx, kernels_of(ctx, pusher)) ? 1 : 0;
     const int fields = ctx->e == ctx->e_a ? 0 : 1;
     cudaGraphExec_t &g = ctx->graph[pusher][parity][sorts ? 1 : 0][late][fields];
     if (!g) {
@@ -1248,27 +1268,38 @@ extern "C" int fetdpic_step(fetdpic_ctx *ctx, long long nsteps, int pusher)
     long long launches = 0;
     const bool timed = ctx->p.time_stages != 0;
     const bool graphs = ctx->p.use_graphs != 0 && !timed && ctx->p.check_interval <= 0;
-    bool begun = false;                          // the previous step's field update carried this one's Faraday
-    for (long long s = 0; s < nsteps; ++s) {
+    const int L = ctx->p.sort_interval;
+    for (long long s = 0; s < nsteps;) {
+        long long run = nsteps - s;              // steps up to the next whole cycle, or the rest
         if (graphs) {
-            const int L = ctx->p.sort_interval;
-            if (L > 1 && ctx->nblocks > 0 && ctx->steps_done % L == 0 && nsteps - s >= L) {
+            if (L > 1 && ctx->nblocks > 0 && ctx->steps_done % L == 0 && run >= L) {
                 rc = cycle_step(ctx, pusher, launches);
                 if (rc) return rc;
-                s += L - 1;
+                s += L;
                 continue;
             }
-            rc = graph_step(ctx, pusher, launches);
-            if (rc) return rc;
-            continue;
+            if (L > 1 && ctx->nblocks > 0) run = std::min<long long>(run, L - ctx->steps_done % L);
+            // a single step is one graph launch; of two or more the field updates are shared, which
+            // plain launches do too (two a step, as fast as the kernels run on the smallest meshes:
+            // 2,048 triangles 10.3 us a step as one-step graphs)
+            if (run == 1) {
+                rc = graph_step(ctx, pusher, launches);
+                if (rc) return rc;
+                ++s;
+                continue;
+            }
         }
-        if (timed && ctx->ev_used > 4000) {
-            CK(cudaStreamSynchronize(ctx->stream));
-            collect_events(ctx);
+        bool begun = false;                      // the previous step's field update carried this one's Faraday
+        for (long long k = 0; k < run; ++k) {
+            if (timed && ctx->ev_used > 4000) {
+                CK(cudaStreamSynchronize(ctx->stream));
+                collect_events(ctx);
+            }
+            const bool more = can_merge(ctx, run - 1 - k);
+            launches += enqueue_step(ctx, pusher, timed, begun, more);
+            begun = more;
         }
-        const bool more = can_merge(ctx, nsteps - 1 - s);
-        launches += enqueue_step(ctx, pusher, timed, begun, more);
-        begun = more;
+        s += run;
     }
     ctx->launches_acc += launches;
     CK(cudaGetLastError());
@@ -1798,7 +1829,7 @@ extern "C" int fetdpic_set_tuning(fetdpic_ctx *ctx, int variant, int sort_interv
     if (!ctx) return FETDPIC_EINVAL;
     if (variant < 0 || variant > 22 || variant == 1 || sort_interval == 0) return ctx->fail(FETDPIC_EINVAL, "bad tuning");
     CK(cudaStreamSynchronize(ctx->stream));
-    ctx->p.kernel_variant = variant == 0 ? FP32_DEFAULT_VARIANT : variant;    // 0 = the untuned default
+    ctx->p.kernel_variant = variant;              // 0 = the untuned default
     ctx->p.sort_interval = sort_interval;
     drop_graphs(ctx);
     return FETDPIC_OK;

@@ -109,6 +109,14 @@ PatchSet build_patches(const PatchInput &in, int T)
     }
     own[np] = seen;
     const int nth = (int)std::max(1u, std::min({16u, std::thread::hardware_concurrency(), (unsigned)((np + 15) / 16)}));
+    if (nth == 1) {
+        PatchSet S;
+        S.soff.assign(1, 0);
+        S.T = T;
+        build_range(S, in, own, T, 0, np);
+        S.ok = np > 0 && S.max_r <= 65535;
+        return S;
+    }
     std::vector<PatchSet> part(nth);
     {
         std::vector<std::thread> th;
@@ -122,6 +130,9 @@ PatchSet build_patches(const PatchInput &in, int T)
     PatchSet S;
     S.soff.assign(1, 0);
     S.T = T;
+    size_t nv = 0, nx = 0, nrow = 0;
+    for (const PatchSet &Q : part) { nv += Q.val.size(); nx += Q.xlist.size(); nrow += Q.row_loc.size(); }
+    S.val.reserve(nv); S.col.reserve(nv); S.xlist.reserve(nx); S.row_loc.reserve(nrow); S.tloc.reserve(4 * (size_t)in.F);
     for (PatchSet &Q : part) {
         const int x = (int)S.xlist.size(), r = (int)S.row_loc.size(), s = (int)S.soff.size() - 1;
         const long long o = (long long)S.col.size() / 2;

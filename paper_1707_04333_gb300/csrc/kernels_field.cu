@@ -225,6 +225,7 @@ size_t field_smem(bool f32, int max_r, int max_e)
 
 cudaError_t field_setup(size_t smem)
 {
+    if (smem <= 48 * 1024) return cudaSuccess;         // what every kernel may use
     cudaError_t e = setup<float, 0, false>(smem);
     if (e == cudaSuccess) e = setup<float, 1, false>(smem);
     if (e == cudaSuccess) e = setup<float, 1, true>(smem);
