@@ -1094,7 +1094,8 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
     else if (f32)
         launch_faraday32(ctx->stream, ctx->F, ctx->csta, ctx->cstb, ctx->dtinv, ctx->e, ctx->b, ctx->rec32, inv2c2, x,
                          ctx->E, ctx->ifix, !timed);
-    else launch_faraday64(ctx->stream, ctx->F, ctx->geo64, ctx->topo, ctx->e, ctx->b, ctx->rec64, ctx->E, ctx->ifix);
+    else launch_faraday64(ctx->stream, ctx->F, ctx->geo64, ctx->topo, ctx->e, ctx->b, ctx->rec64, ctx->E, ctx->ifix,
+                          !timed);
     launches += ctx->F > 0 && !begun;
     if (timed) mark(ctx, 0);
     if (check && !ctx->q_prev_valid) { charge_now(ctx, ctx->q0); launches += 2; }
@@ -1104,7 +1105,11 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
             a.pdl = !timed;
             launch_particles32(ctx->stream, pusher, a);
         }
-        else launch_particles64(ctx->stream, pusher, args64(ctx));
+        else {
+            StepArgs64 a = args64(ctx);
+            a.pdl = !timed;
+            launch_particles64(ctx->stream, pusher, a);
+        }
         ++launches;
     }
     if (timed) mark(ctx, 1);

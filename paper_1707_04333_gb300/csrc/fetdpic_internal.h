@@ -239,6 +239,7 @@ struct StepArgs64 {
     const int *id;                          // load index of each particle slot
     const int *edge_off;                    // per instance, for instance-local record ids
     long long nchunks; int block;
+    bool pdl;                               // programmatic dependent launch (launch_k)
     bool soft;                              // geometry and species constants suit the integer arithmetic
     bool ext_on;                            // some applied field or profile is set
     const signed char *tshift;              // [F][3] periodic shift codes; NULL = no periodic walls
@@ -267,7 +268,7 @@ struct StepArgs32 {
 // The Faraday launches also clear the current accumulator (ifix, E edges) for
 // the particle kernel after them.
 void launch_faraday64(cudaStream_t st, int F, const Geo64 *geo, const Topo *topo, const double *e,
-                      double *b, Rec64 *rec, int E, unsigned long long *ifix);
+                      double *b, Rec64 *rec, int E, unsigned long long *ifix, bool pdl);
 // Applied fields folded into the FP32 field record (ext == NULL: none): per
 // instance (E_x, E_y, B_z, 0) times the amplitude (E) and the per-triangle
 // weights extw (NULL = 1); finst = instance of each triangle.

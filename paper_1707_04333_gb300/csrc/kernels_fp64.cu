@@ -21,34 +21,41 @@ __global__ void k_faraday64(int F, const Geo64 *__restrict__ geo, const Topo *__
                             unsigned long long *__restrict__ ifix)
 {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
+    int3 w{};
+    double dt = 0.0, inv2A = 0.0;
+    if (f < F) {
+        // static, loaded before the wait for the kernel that writes e
+        w = make_int3(topo[f].ew[0], topo[f].ew[1], topo[f].ew[2]);
+        dt = geo[f].dt; inv2A = geo[f].inv2A;
+    }
+    pdl_begin();
     for (int k = f; k < E; k += gridDim.x * blockDim.x) ifix[k] = 0ull;      // for the particle kernel
     if (f >= F) return;
-    const Topo t = topo[f];
+    const int ew[3] = {w.x, w.y, w.z};
     double se[3];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-        const double v = e[t.ew[m] >> 1];
-        se[m] = (t.ew[m] & 1) ? -v : v;
+        const double v = e[ew[m] >> 1];
+        se[m] = (ew[m] & 1) ? -v : v;
     }
     double ce = 0.0;
     ce = ce + se[0];
     ce = ce + se[1];
     ce = ce + se[2];
     const double bo = b[f];
-    const double dt = geo[f].dt;
     const double bn = bo - dt * ce;
     b[f] = bn;
     Rec64 r;
     r.se[0] = se[0]; r.se[1] = se[1]; r.se[2] = se[2];
-    r.bz = (bn + bo) * geo[f].inv2A;
+    r.bz = (bn + bo) * inv2A;
     rec[f] = r;
 }
 
 void launch_faraday64(cudaStream_t st, int F, const Geo64 *geo, const Topo *topo, const double *e,
-                      double *b, Rec64 *rec, int E, unsigned long long *ifix)
+                      double *b, Rec64 *rec, int E, unsigned long long *ifix, bool pdl)
 {
     if (F <= 0) return;
-    k_faraday64<<<(F + 255) / 256, 256, 0, st>>>(F, geo, topo, e, b, rec, E, ifix);
+    launch_k(pdl, k_faraday64, dim3((F + 255) / 256), dim3(256), st, F, geo, topo, e, b, rec, E, ifix);
 }
 
 // ------------------------------------------------------------ arithmetic
@@ -450,6 +457,7 @@ __device__ __forceinline__ void walk64_any(const StepArgs64 &a, const Walk64 *it
 template <int PUSHER>
 __global__ void __launch_bounds__(256, 2) k_particles64(StepArgs64 a)
 {
+    pdl_begin();
     extern __shared__ Walk64 rings[];
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -538,9 +546,14 @@ static void launch_p64(cudaStream_t st, const StepArgs64 &a)
         dev = d; blk = a.block;
         if (per_sm < 1) per_sm = 1;
     }
-    const long long nw = a.block / 32, need = (a.nchunks + nw - 1) / nw;
+    // few chunks go to as many SMs as there are, in blocks of fewer warps (4,000 particles: 125 chunks
+    // in 16 blocks of 8 warps left 136 SMs idle)
+    long long nw = (a.nchunks + sms - 1) / sms;
+    if (nw > a.block / 32) nw = a.block / 32;
+    const long long need = (a.nchunks + nw - 1) / nw;
     const long long grid = need < (long long)per_sm * sms ? need : (long long)per_sm * sms;
-    k_particles64<PUSHER><<<(unsigned)grid, a.block, ring, st>>>(a);
+    launch_ks(a.pdl, k_particles64<PUSHER>, dim3((unsigned)grid), dim3((unsigned)nw * 32),
+              (size_t)nw * RING64 * sizeof(Walk64), st, a);
 }
 
 void launch_particles64(cudaStream_t st, int pusher, const StepArgs64 &a)
