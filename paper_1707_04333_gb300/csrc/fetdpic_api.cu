@@ -118,6 +118,8 @@ struct fetdpic_ctx {
     unsigned long long *q0 = nullptr, *q1 = nullptr;
     double *g0 = nullptr, *qunit = nullptr, *chk_out = nullptr, *eng_part = nullptr;
     long long *h_rp = nullptr; int *h_ci = nullptr; double *h_v = nullptr;
+    unsigned *chk_ticket = nullptr;           // blocks of the check kernel that are done
+    bool q1_clean = false;                    // q1 is zero (cleared by the last check)
     bool q_prev_valid = false;                // q0 holds the charge of the current particle state
     bool g0_ready = false;
     std::vector<char> gauss_abs;              // per instance: Gauss law checked absolutely (after the solve)
@@ -595,7 +597,8 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
             ctx->g0 = ctx->alloc<double>(ctx->N);
             ctx->qunit = ctx->alloc<double>(n_inst);
             ctx->chk_out = ctx->alloc<double>(3 * (size_t)n_inst);
-            ctx->eng_part = ctx->alloc<double>((size_t)energy_blocks(ctx->E, ctx->F) * n_inst);
+            ctx->eng_part = ctx->alloc<double>((size_t)check_blocks(ctx->N, ctx->E, ctx->F) * n_inst);
+            ctx->chk_ticket = ctx->alloc<unsigned>(1);
             ctx->h_rp = ctx->alloc<long long>(hrp.size());
             ctx->h_ci = ctx->alloc<int>(hci.size());
             ctx->h_v = ctx->alloc<double>(hv.size());
@@ -613,6 +616,7 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         rc = rc ? rc : upload(ctx, ctx->h_v, hv.data(), hv.size());
         if (rc) return rc;
         CK(cudaMemsetAsync(ctx->chk_out, 0, sizeof(double) * 3 * n_inst, ctx->stream));
+        CK(cudaMemsetAsync(ctx->chk_ticket, 0, sizeof(unsigned), ctx->stream));
     }
     rc = rc ? rc : upload(ctx, ctx->geo64, g64.data(), g64.size());
     if (!g32.empty()) rc = rc ? rc : upload(ctx, ctx->csta, g32.data(), g32.size());
@@ -709,10 +713,10 @@ extern "C" int fetdpic_load_particles(fetdpic_ctx *ctx, int inst, double q, doub
 }
 
 // Charge of the current particle state into q (fixed point).
-static void charge_now(fetdpic_ctx *ctx, unsigned long long *q)
+static void charge_now(fetdpic_ctx *ctx, unsigned long long *q, bool clean = false, bool pdl = false)
 {
     launch_charge(ctx->stream, ctx->p.precision == FETDPIC_FP32, ctx->P, ctx->cell, ctx->chunk_sp, ctx->sp_dev,
-                  ctx->geo64, ctx->topo, ctx->f[0], ctx->f[1], q, ctx->N);
+                  ctx->geo64, ctx->topo, ctx->f[0], ctx->f[1], q, ctx->N, clean, pdl);
 }
 
 // The Gauss-law check compares S~ d - q with its value at this point (after
@@ -721,8 +725,7 @@ static void reset_gauss_reference(fetdpic_ctx *ctx)
 {
     if (!ctx->g0 || !ctx->finalized) { ctx->q_prev_valid = false; return; }
     charge_now(ctx, ctx->q0);
-    launch_dgl(ctx->stream, ctx->N, ctx->nrp, ctx->nedge, ctx->ninst, ctx->qunit, ctx->d, ctx->q0, ctx->g0, 1,
-               ctx->chk_out);
+    launch_gauss_reference(ctx->stream, ctx->N, ctx->nrp, ctx->nedge, ctx->ninst, ctx->qunit, ctx->d, ctx->q0, ctx->g0);
     // after the electrostatic solve the reference is zero off the PEC walls: S~ d^n = q^n itself is
     // checked there; on wall nodes S~ d - q is the conductor's induced charge and stays relative
     for (size_t k = 0; k < ctx->gauss_abs.size(); ++k) {
@@ -1048,17 +1051,17 @@ static void swap_fields(fetdpic_ctx *ctx)
     std::swap(ctx->ifix, ctx->ifix_alt);
 }
 
-// Whether the step that `after` more steps follow may share its field update with
-// the next: Ampere's of one step with Faraday's of the next (not with stage events,
-// whose stages are separate; not the step of a check, which looks at the fields
-// between them).
+// Whether a step computes the conservation checks.
 static bool checks_at(const fetdpic_ctx *ctx, long long step)
 {
     return ctx->p.check_interval > 0 && ctx->g0 && step % ctx->p.check_interval == 0;
 }
+// Whether the step that `after` more steps follow may share its field update with
+// the next: Ampere's of one step with Faraday's of the next (not with stage events,
+// whose stages are separate).
 static bool can_merge(const fetdpic_ctx *ctx, long long after)
 {
-    return after > 0 && ctx->patches && ctx->p.time_stages == 0 && !checks_at(ctx, ctx->steps_done + 1);
+    return after > 0 && ctx->patches && ctx->p.time_stages == 0;
 }
 
 // One time step: Faraday (+ field record), particles, Ampere, periodic sort.
@@ -1098,7 +1101,7 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
                           !timed);
     launches += ctx->F > 0 && !begun;
     if (timed) mark(ctx, 0);
-    if (check && !ctx->q_prev_valid) { charge_now(ctx, ctx->q0); launches += 2; }
+    if (check && !ctx->q_prev_valid) { charge_now(ctx, ctx->q0, false, !timed); launches += 1; }
     if (ctx->nblocks > 0) {
         if (f32) {
             StepArgs32 a = args32(ctx, pusher);
@@ -1126,9 +1129,8 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
         cudaEventRecord(ctx->ev_join, ctx->side);
     }
     if (check) {
-        charge_now(ctx, ctx->q1);
-        launch_dce(ctx->stream, ctx->N, ctx->nrp, ctx->nedge, ctx->ninst, ctx->ifix, ctx->q0, ctx->q1, ctx->chk_out);
-        launches += 3;
+        charge_now(ctx, ctx->q1, ctx->q1_clean, !timed);
+        ++launches;
     }
     if (ctx->patches) {
         FieldArgs W = ctx->field;
@@ -1158,11 +1160,19 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
     }
     if (timed) mark(ctx, 3);
     if (check) {
-        launch_dgl(ctx->stream, ctx->N, ctx->nrp, ctx->nedge, ctx->ninst, ctx->qunit, ctx->d, ctx->q1, ctx->g0, 0,
-                   ctx->chk_out);
-        launch_energy(ctx->stream, ctx->E, ctx->F, ctx->h_rp, ctx->h_ci, ctx->h_v, ctx->e, ctx->einst, ctx->b,
-                      ctx->geo64, ctx->topo, (int)ctx->mesh.size(), ctx->eng_part, ctx->chk_out);
-        launches += 3;
+        CheckArgs C{};
+        C.N = ctx->N; C.E = ctx->E; C.F = ctx->F; C.ninst_n = (int)ctx->mesh.size();
+        C.nrp = ctx->nrp; C.nedge = ctx->nedge; C.ninst = ctx->ninst;
+        // after a field update that carried the next Faraday, this step's current and b are in the
+        // other buffers (and stay there until the next field update)
+        C.ifix = more ? ctx->ifix_alt : ctx->ifix;
+        C.b = more ? ctx->b_alt : ctx->b;
+        C.q0 = ctx->q0; C.q1 = ctx->q1; C.qunit = ctx->qunit; C.d = ctx->d; C.g0 = ctx->g0;
+        C.hrp = ctx->h_rp; C.hci = ctx->h_ci; C.hv = ctx->h_v;
+        C.e = ctx->e; C.einst = ctx->einst; C.geo = ctx->geo64; C.topo = ctx->topo;
+        C.part = ctx->eng_part; C.out = ctx->chk_out; C.ticket = ctx->chk_ticket;
+        launches += launch_checks(ctx->stream, C, !timed);
+        ctx->q1_clean = true;                 // q0, cleared, becomes q1
         std::swap(ctx->q0, ctx->q1);          // the charge after this step is the next step's q^n
         ctx->q_prev_valid = true;
         if (timed) mark(ctx, 5);

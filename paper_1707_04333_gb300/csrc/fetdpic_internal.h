@@ -350,22 +350,30 @@ void launch_sort(cudaStream_t st, const SortArgs &a);
 
 
 // Conservation checks (kernels_check.cu).
+// `clean`: q is zero already.
 void launch_charge(cudaStream_t st, bool fp32, long long P, const int *cell, const short *chunk_sp, const Species *sp,
-                   const Geo64 *geo, const Topo *topo, const void *f0, const void *f1, unsigned long long *q, int N);
-void launch_dce(cudaStream_t st, int N, const int *nrp, const int *nedge, const int *ninst,
-                const unsigned long long *ifix, const unsigned long long *q0, const unsigned long long *q1, double *out);
+                   const Geo64 *geo, const Topo *topo, const void *f0, const void *f1, unsigned long long *q, int N,
+                   bool clean, bool pdl);
+void launch_gauss_reference(cudaStream_t st, int N, const int *nrp, const int *nedge, const int *ninst,
+                            const double *qunit, const double *d, const unsigned long long *q, double *g0);
+struct CheckArgs {
+    int N, E, F, ninst_n;
+    const int *nrp, *nedge, *ninst;          // node -> edges (edge << 1 | enters the node), instance of each node
+    const unsigned long long *ifix;           // the step's current
+    unsigned long long *q0; const unsigned long long *q1;   // charge before (cleared) and after the step
+    const double *qunit, *d, *g0;
+    const long long *hrp; const int *hci; const double *hv; // full [*eps]
+    const double *e; const int *einst; const double *b; const Geo64 *geo; const Topo *topo;
+    double *part, *out;                      // partial energies; (dce, dgl, energy) per instance
+    unsigned *ticket;                        // blocks done, zero between launches
+};
+int launch_checks(cudaStream_t st, const CheckArgs &a, bool pdl);       // kernels launched
+long long check_blocks(int N, int E, int F);
 // Field probe: E(x_p) = sum_m w_m e[eg_m], w_m = s_m (l_a grad l_b - l_b grad l_a)
 // at the probe's barycentrics (a = m+1, b = m+2), precomputed on the host.
 struct ProbeW { double w[6]; int eg[3]; int pad; };
 void launch_probe(cudaStream_t st, long long n, const ProbeW *pw, const double *e, double2 *ring, long long cap,
                   unsigned long long *count);
-void launch_dgl(cudaStream_t st, int N, const int *nrp, const int *nedge, const int *ninst, const double *qunit,
-                const double *d, const unsigned long long *q, double *g0, int init, double *out);
-long long energy_blocks(int E, int F);
-void launch_energy(cudaStream_t st, int E, int F, const long long *hrp, const int *hci, const double *hv,
-                   const double *e, const int *einst, const double *b, const Geo64 *geo, const Topo *topo,
-                   int ninst, double *part, double *out);
-
 size_t scan_tmp_ints(long long n);
 void launch_exclusive_scan(cudaStream_t st, const int *in, int *out, long long n, int *tmp);
 

@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(256) k_charge64(long long nchunks, const int *
                                                   const double *__restrict__ x, const double *__restrict__ y,
                                                   unsigned long long *__restrict__ q)
 {
+    pdl_begin();
     const int lane = threadIdx.x & 31;
     const long long ch = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (ch >= nchunks) return;
@@ -86,6 +87,7 @@ __global__ void __launch_bounds__(256) k_charge32(long long nchunks, const int *
                                                   const Topo *__restrict__ topo, const float *__restrict__ l0,
                                                   const float *__restrict__ l1, unsigned long long *__restrict__ q)
 {
+    pdl_begin();
     const int lane = threadIdx.x & 31;
     const long long c0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * CH_CHUNKS;
     int f[CH_CHUNKS];
@@ -154,49 +156,22 @@ __device__ __forceinline__ void warp_max_pos(double *out, int slot, int in, doub
 // Edges of a node whose values are loaded before any is summed (in order).
 constexpr int NB = 8;
 
-// Continuity residual per node: res = (q1 - q0) + sum_e o(k,e) i_e, exactly in
-// integers; normalised by sum_e |i_e| + |q1 - q0| (at least one unit).
-__global__ void k_dce(int N, const int *__restrict__ nrp, const int *__restrict__ nedge,
-                      const int *__restrict__ ninst, const unsigned long long *__restrict__ ifix,
-                      const unsigned long long *__restrict__ q0, const unsigned long long *__restrict__ q1,
-                      double *__restrict__ out)
+// One instance's energy: a warp sums the block partials, in an order that depends on their number only.
+__device__ __forceinline__ void energy_sum(long long nblocks, int ninst, const double *part, int in, int lane, double *out)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = k < N;
-    long long flux = 0;
-    double absf = 0.0;
-    for (int r = live ? nrp[k] : 0, r1 = live ? nrp[k + 1] : 0; r < r1; r += NB) {
-        int w[NB];
-        long long iv[NB];
+    double s = 0.0;
+    for (long long k = lane; k < nblocks; k += 32) s += __ldcg(part + k * ninst + in);
 #pragma unroll
-        for (int i = 0; i < NB; ++i) w[i] = r + i < r1 ? nedge[r + i] : 0;
-#pragma unroll
-        for (int i = 0; i < NB; ++i) iv[i] = r + i < r1 ? (long long)ifix[w[i] >> 1] : 0;
-#pragma unroll
-        for (int i = 0; i < NB; ++i)
-            if (r + i < r1) {
-                flux += (w[i] & 1) ? -iv[i] : iv[i];
-                absf += fabs((double)iv[i]);
-            }
-    }
-    const long long dq = live ? (long long)q1[k] - (long long)q0[k] : 0;
-    const long long res = dq + flux;
-    const double scale = fmax(absf + fabs((double)dq), 1.0);
-    warp_max_pos(out, 0, live ? ninst[k] : 0, fabs((double)res) / scale, live);
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) out[3 * in + 2] = s;
 }
 
-// Gauss residual per node: g = sum_e o(k,e) d_e - q (physical units).  With
-// init != 0 it stores g as the reference g0; otherwise it reports
-// |g - g0| / (sum |d_e| + |q| + |g0|).
-__global__ void k_dgl(int N, const int *__restrict__ nrp, const int *__restrict__ nedge,
-                      const int *__restrict__ ninst, const double *__restrict__ qunit,
-                      const double *__restrict__ d, const unsigned long long *__restrict__ q,
-                      double *__restrict__ g0, int init, double *__restrict__ out)
+// Node k's sums over its edges: Gauss sum_e o(k,e) d_e and sum_e |d_e|.
+__device__ __forceinline__ void node_flux(const int *__restrict__ nrp, const int *__restrict__ nedge,
+                                          const double *__restrict__ d, int k, double &s, double &sa)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = k < N;
-    double s = 0.0, sa = 0.0;
-    for (int r = live ? nrp[k] : 0, r1 = live ? nrp[k + 1] : 0; r < r1; r += NB) {
+    s = 0.0; sa = 0.0;
+    for (int r = nrp[k], r1 = nrp[k + 1]; r < r1; r += NB) {
         int w[NB];
         double v[NB];
 #pragma unroll
@@ -210,46 +185,88 @@ __global__ void k_dgl(int N, const int *__restrict__ nrp, const int *__restrict_
                 sa += fabs(v[i]);
             }
     }
-    const int in = live ? ninst[k] : 0;
-    const double qk = live ? (double)(long long)q[k] * qunit[in] : 0.0;
-    const double g = s - qk;
-    if (init) { if (live) g0[k] = g; return; }
-    const double ref = live ? g0[k] : 0.0;
-    const double scale = sa + fabs(qk) + fabs(ref);
-    const double nr = scale > 0.0 ? fabs(g - ref) / scale : 0.0;
-    warp_max_pos(out, 1, in, nr, live);
 }
 
-// Energy, first pass: per block, sum over its edges of e_k ([*eps] e)_k / 2 and
-// over its faces of b_f^2 / (2 mu0 A_f), per instance; written to part[block].
-__global__ void k_energy_part(int E, int F, const long long *__restrict__ hrp, const int *__restrict__ hci,
-                              const double *__restrict__ hv, const double *__restrict__ e,
-                              const int *__restrict__ einst, const double *__restrict__ b,
-                              const Geo64 *__restrict__ geo, const Topo *__restrict__ topo,
-                              int ninst, double *__restrict__ part)
+// The Gauss-law reference g0 = sum_e o(k,e) d_e - q (physical units).
+__global__ void __launch_bounds__(256) k_gauss_reference(int N, const int *__restrict__ nrp,
+                                                         const int *__restrict__ nedge, const int *__restrict__ ninst,
+                                                         const double *__restrict__ qunit, const double *__restrict__ d,
+                                                         const unsigned long long *__restrict__ q, double *__restrict__ g0)
 {
-    extern __shared__ double sh[];              // [blockDim.x]
-    __shared__ int lo_s, hi_s;
-    const int tid = threadIdx.x;
-    const long long i = (long long)blockIdx.x * blockDim.x + tid;
-    const bool edge = i < E, face = i < F;
-    const int ie = edge ? einst[i] : -1, jf = face ? topo[i].inst : -1;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= N) return;
+    double s, sa;
+    node_flux(nrp, nedge, d, k, s, sa);
+    const double qk = (double)(long long)q[k] * qunit[ninst[k]];
+    g0[k] = s - qk;
+}
+
+// The checks of a step in one launch (they were four, each a short wave with a
+// gap before it), thread i for node i, edge i and face i:
+//   - continuity residual of node i: res = (q1 - q0) + sum_e o(k,e) i_e, exactly
+//     in integers, over sum_e |i_e| + |q1 - q0| (at least one unit), the largest
+//     per instance;
+//   - Gauss residual |g - g0| / (sum |d_e| + |q| + |g0|) with g = sum_e o(k,e)
+//     d_e - q, the largest per instance;
+//   - energy: per block and instance the sum of e_k ([*eps] e)_k / 2 over its
+//     edges and b_f^2 / (2 mu0 A_f) over its faces, in `part`, summed by the
+//     last block (`ticket`; few partials) or by k_energy_final.
+// q0, the charge before the step, is not needed any more: it is cleared for the
+// next charge.
+__global__ void __launch_bounds__(256) k_checks(CheckArgs a)
+{
+    pdl_begin();
+    __shared__ double sh[256];
+    __shared__ int lo_s, hi_s, last_s;
+    const int tid = threadIdx.x, i = blockIdx.x * 256 + tid;
+    {
+        const bool live = i < a.N;
+        long long flux = 0;
+        double absf = 0.0, s = 0.0, sa = 0.0;
+        if (live) {
+            for (int r = a.nrp[i], r1 = a.nrp[i + 1]; r < r1; r += NB) {
+                int w[NB];
+                long long iv[NB];
+#pragma unroll
+                for (int k = 0; k < NB; ++k) w[k] = r + k < r1 ? a.nedge[r + k] : 0;
+#pragma unroll
+                for (int k = 0; k < NB; ++k) iv[k] = r + k < r1 ? (long long)a.ifix[w[k] >> 1] : 0;
+#pragma unroll
+                for (int k = 0; k < NB; ++k)
+                    if (r + k < r1) {
+                        flux += (w[k] & 1) ? -iv[k] : iv[k];
+                        absf += fabs((double)iv[k]);
+                    }
+            }
+            node_flux(a.nrp, a.nedge, a.d, i, s, sa);
+        }
+        const int in = live ? a.ninst[i] : 0;
+        const long long q1 = live ? (long long)a.q1[i] : 0, dq = live ? q1 - (long long)a.q0[i] : 0;
+        if (live) a.q0[i] = 0ull;
+        const double scale = fmax(absf + fabs((double)dq), 1.0);
+        warp_max_pos(a.out, 0, in, fabs((double)(dq + flux)) / scale, live);
+        const double qk = live ? (double)q1 * a.qunit[in] : 0.0, ref = live ? a.g0[i] : 0.0;
+        const double g = s - qk, gs = sa + fabs(qk) + fabs(ref);
+        warp_max_pos(a.out, 1, in, gs > 0.0 ? fabs(g - ref) / gs : 0.0, live);
+    }
+    const bool edge = i < a.E, face = i < a.F;
+    const int ie = edge ? a.einst[i] : -1, jf = face ? a.topo[i].inst : -1;
     double ve = 0.0, vf = 0.0;
     if (edge) {
         double s = 0.0;
-        for (long long q = hrp[i]; q < hrp[i + 1]; ++q) s += hv[q] * e[hci[q]];
-        ve = 0.5 * e[i] * s;
+        for (long long q = a.hrp[i]; q < a.hrp[i + 1]; ++q) s += a.hv[q] * a.e[a.hci[q]];
+        ve = 0.5 * a.e[i] * s;
     }
-    if (face) vf = 0.5 * b[i] * b[i] * geo[i].hb;
+    if (face) vf = 0.5 * a.b[i] * a.b[i] * a.geo[i].hb;
     // the instances this block holds part of: usually one
-    if (tid == 0) { lo_s = ninst; hi_s = -1; }
+    if (tid == 0) { lo_s = a.ninst_n; hi_s = -1; }
     __syncthreads();
     if (edge) { atomicMin(&lo_s, ie); atomicMax(&hi_s, ie); }
     if (face) { atomicMin(&lo_s, jf); atomicMax(&hi_s, jf); }
     __syncthreads();
     const int lo = lo_s, hi = hi_s;
-    double *out = part + (long long)blockIdx.x * ninst;
-    for (int in = tid; in < ninst; in += blockDim.x)
+    double *out = a.part + (long long)blockIdx.x * a.ninst_n;
+    for (int in = tid; in < a.ninst_n; in += 256)
         if (in < lo || in > hi) out[in] = 0.0;
     for (int in = lo; in <= hi; ++in) {
         double v = 0.0;
@@ -257,64 +274,61 @@ __global__ void k_energy_part(int E, int F, const long long *__restrict__ hrp, c
         if (jf == in) v += vf;
         sh[tid] = v;
         __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+        for (int o = 128; o > 0; o >>= 1) {
             if (tid < o) sh[tid] += sh[tid + o];
             __syncthreads();
         }
         if (tid == 0) out[in] = sh[0];
         __syncthreads();
     }
+    if (!a.ticket) return;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last_s = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last_s) return;
+    if (tid == 0) *a.ticket = 0u;
+    for (int in = tid >> 5; in < a.ninst_n; in += 8) energy_sum(gridDim.x, a.ninst_n, a.part, in, tid & 31, a.out);
 }
 
-// Energy, second pass: one warp per instance sums the block partials, in an order
-// that depends on their number only.
+// Energy, second pass for many partials: one warp per instance.
 __global__ void k_energy_final(long long nblocks, int ninst, const double *__restrict__ part, double *__restrict__ out)
 {
-    const int in = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (in >= ninst) return;
-    double s = 0.0;
-    for (long long k = lane; k < nblocks; k += 32) s += part[k * ninst + in];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) out[3 * in + 2] = s;
+    const int in = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (in < ninst) energy_sum(nblocks, ninst, part, in, threadIdx.x & 31, out);
 }
 
 void launch_charge(cudaStream_t st, bool fp32, long long P, const int *cell, const short *chunk_sp, const Species *sp,
-                   const Geo64 *geo, const Topo *topo, const void *f0, const void *f1, unsigned long long *q, int N)
+                   const Geo64 *geo, const Topo *topo, const void *f0, const void *f1, unsigned long long *q, int N,
+                   bool clean, bool pdl)
 {
-    cudaMemsetAsync(q, 0, sizeof(unsigned long long) * (size_t)N, st);
+    if (!clean) cudaMemsetAsync(q, 0, sizeof(unsigned long long) * (size_t)N, st);
     if (P <= 0) return;
     const long long nch = P / 32, warps = fp32 ? (nch + CH_CHUNKS - 1) / CH_CHUNKS : nch;
-    const unsigned g = (unsigned)((warps + 7) / 8);
-    if (fp32) k_charge32<<<g, 256, 0, st>>>(nch, cell, chunk_sp, sp, topo, (const float *)f0, (const float *)f1, q);
-    else k_charge64<<<g, 256, 0, st>>>(nch, cell, chunk_sp, sp, geo, topo, (const double *)f0, (const double *)f1, q);
+    const dim3 g((unsigned)((warps + 7) / 8));
+    if (fp32) launch_k(pdl, k_charge32, g, dim3(256), st, nch, cell, chunk_sp, sp, topo, (const float *)f0, (const float *)f1, q);
+    else launch_k(pdl, k_charge64, g, dim3(256), st, nch, cell, chunk_sp, sp, geo, topo, (const double *)f0, (const double *)f1, q);
 }
 
-void launch_dce(cudaStream_t st, int N, const int *nrp, const int *nedge, const int *ninst,
-                const unsigned long long *ifix, const unsigned long long *q0, const unsigned long long *q1, double *out)
+void launch_gauss_reference(cudaStream_t st, int N, const int *nrp, const int *nedge, const int *ninst,
+                            const double *qunit, const double *d, const unsigned long long *q, double *g0)
 {
-    if (N <= 0) return;
-    k_dce<<<(N + 255) / 256, 256, 0, st>>>(N, nrp, nedge, ninst, ifix, q0, q1, out);
+    if (N > 0) k_gauss_reference<<<(N + 255) / 256, 256, 0, st>>>(N, nrp, nedge, ninst, qunit, d, q, g0);
 }
 
-void launch_dgl(cudaStream_t st, int N, const int *nrp, const int *nedge, const int *ninst, const double *qunit,
-                const double *d, const unsigned long long *q, double *g0, int init, double *out)
-{
-    if (N <= 0) return;
-    k_dgl<<<(N + 255) / 256, 256, 0, st>>>(N, nrp, nedge, ninst, qunit, d, q, g0, init, out);
-}
+long long check_blocks(int N, int E, int F) { return ((long long)std::max(N, std::max(E, F)) + 255) / 256; }
 
-long long energy_blocks(int E, int F) { return ((long long)(E > F ? E : F) + 255) / 256; }
-
-void launch_energy(cudaStream_t st, int E, int F, const long long *hrp, const int *hci, const double *hv,
-                   const double *e, const int *einst, const double *b, const Geo64 *geo, const Topo *topo,
-                   int ninst, double *part, double *out)
+int launch_checks(cudaStream_t st, const CheckArgs &a, bool pdl)
 {
-    const long long nb = energy_blocks(E, F);
-    if (nb <= 0) return;
-    k_energy_part<<<(unsigned)nb, 256, 256 * sizeof(double), st>>>(E, F, hrp, hci, hv, e, einst, b, geo, topo, ninst,
-                                                                    part);
-    k_energy_final<<<(ninst + 7) / 8, 256, 0, st>>>(nb, ninst, part, out);
+    const long long nb = check_blocks(a.N, a.E, a.F);
+    if (nb <= 0) return 0;
+    CheckArgs w = a;
+    // one block sums the partials as fast as a launch would start; many are spread over more warps
+    const bool own = nb * a.ninst_n <= 16384;
+    if (!own) w.ticket = nullptr;
+    launch_k(pdl, k_checks, dim3((unsigned)nb), dim3(256), st, w);
+    if (!own) k_energy_final<<<(a.ninst_n + 7) / 8, 256, 0, st>>>(nb, a.ninst_n, a.part, a.out);
+    return own ? 1 : 2;
 }
 
 
