@@ -85,6 +85,7 @@ struct fetdpic_ctx {
     Sp32 *sp32_dev = nullptr;
     int sms = 0;                             // of the device
     bool soft64 = false;                     // FP64 constants within the integer arithmetic's range
+    double density = 0.0;                    // particles per triangle where the particles are
     long long P = 0, nblocks = 0;
     int block = 256;
     int *cell = nullptr, *cell_tmp = nullptr, *id = nullptr, *id_tmp = nullptr;
@@ -813,6 +814,13 @@ static int finalize(fetdpic_ctx *ctx)
         hist_n += D.nf + 1;                  // the species' triangles, then its padding bin
         off += D.cap;
     }
+    {
+        std::vector<double> n(ni, 0.0);
+        for (const Species &D : ctx->sp) n[D.inst] += (double)D.n;
+        double all = 0.0, sum = 0.0;
+        for (int k = 0; k < ni; ++k) { all += n[k]; sum += n[k] * (n[k] / ctx->mesh[k].nf); }
+        ctx->density = all > 0.0 ? sum / all : 0.0;
+    }
     ctx->soft64 = true;
     for (const Species &D : ctx->sp)
         ctx->soft64 = ctx->soft64 && soft_constant(D.alpha) && soft_constant(D.ic2) && soft_constant(D.dt) &&
@@ -956,7 +964,9 @@ static constexpr Hybrid HYBRIDS[] = {{17, 12, 14, 6}, {18, 12, 14, 4}, {21, 19, 
 //     (64 particles: 6.15 against 6.7 with variant 22; 4,000: 7.0 against 7.6; with two chunks per
 //     SM variant 12 is ahead, 8.72 against 8.93);
 //   - fewer than twelve particles per triangle: runs are short from the start and the window's flush
-//     does not pay (two per triangle: 42.5 with variant 12, 44.7 with 22; eight: 18.7 against 20.1);
+//     does not pay (two per triangle: 42.5 with variant 12, 44.7 with 22; eight: 18.7 against 20.1).
+//     Counted where the particles are, since a batch may be uneven (16 instances with 2 to 96 per
+//     triangle, 6.8 in all but 30 around the mean particle: 53.9 with the window kernels, 56.6 without);
 //   - else an early and a late kernel.  Early, 28 warps per SM for the Vay pusher, 24 for the others,
 //     whose kernels spill at 72 registers (8 M particles, Higuera-Cary: 130.5 against 134.3).  Late, the 20-warp window kernel up to 2 M particles,
 //     where its few more particles per warp cost less than registers held back from it (1.1 M in 16
@@ -969,7 +979,7 @@ static Hybrid kernels_of(const fetdpic_ctx *ctx, int pusher)
     if (v != 0) return Hybrid{v, v, v, 0};
     const long long n64 = ctx->P / 64;
     if (n64 <= ctx->sms) return Hybrid{0, 4, 4, 0};
-    if (ctx->P < 12ll * ctx->F) return Hybrid{0, 12, 12, 0};
+    if (ctx->density < 12.0) return Hybrid{0, 12, 12, 0};
     return Hybrid{0, pusher == FETDPIC_VAY ? 19 : 12, n64 < 32768 ? 14 : 20, 6};
 }
 
