@@ -1036,6 +1036,25 @@ static void collect_events(fetdpic_ctx *ctx)
     ctx->ev_used = 0;
 }
 
+static void swap_particles(fetdpic_ctx *ctx)
+{
+    std::swap(ctx->cell, ctx->cell_tmp);
+    std::swap(ctx->id, ctx->id_tmp);
+    for (int k = 0; k < 4; ++k) std::swap(ctx->f[k], ctx->f_tmp[k]);
+}
+
+// Up to this many slots are not sorted: no result depends on the order, a few warps gain nothing from it,
+// and its four launches and their join take 0.6 us of a step (us a step with a sort every 16 and without,
+// 2,048 triangles: 64 particles 6.07 and 5.50, 1,024 6.87 and 6.28, 2,048 7.06 and 6.41).  At 4,096 particles
+// the two are even (7.26 and 7.19); at 8,192 scattered ones lose (7.33 and 8.66).
+constexpr long long SORT_MIN_SLOTS = 2048;
+
+// Whether step `step` (from 1) ends with a sort.
+static bool sorts_at(const fetdpic_ctx *ctx, long long step)
+{
+    return ctx->p.sort_interval > 0 && ctx->P > SORT_MIN_SLOTS && step % ctx->p.sort_interval == 0;
+}
+
 static void do_sort(fetdpic_ctx *ctx, cudaStream_t st)
 {
     SortArgs s{};
@@ -1047,9 +1066,7 @@ static void do_sort(fetdpic_ctx *ctx, cudaStream_t st)
     s.hist = ctx->hist; s.hoff = ctx->hoff; s.hist_n = ctx->hist_n; s.scan_tmp = ctx->scan_tmp;
     s.chunk_sp = ctx->chunk_sp;
     launch_sort(st, s);
-    std::swap(ctx->cell, ctx->cell_tmp);
-    std::swap(ctx->id, ctx->id_tmp);
-    for (int k = 0; k < 4; ++k) std::swap(ctx->f[k], ctx->f_tmp[k]);
+    swap_particles(ctx);
 }
 
 // The buffers of e, b and the current accumulator change places (a field update
@@ -1126,21 +1143,22 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
         ++launches;
     }
     if (timed) mark(ctx, 1);
-    // the sort of this step's end reads only the particle state, which the Ampere update
-    // does not touch: without stage events or checks it runs on the side stream meanwhile
-    const bool sorts = ctx->p.sort_interval > 0 && ctx->nblocks > 0 &&
-                       (ctx->steps_done + 1) % ctx->p.sort_interval == 0;
-    const bool side_sort = sorts && !timed && !check;
+    if (check) {
+        charge_now(ctx, ctx->q1, ctx->q1_clean, !timed);
+        ++launches;
+    }
+    // the sort of this step's end reads only the particle state, which the field update and the
+    // checks after the charge do not touch: without stage events it runs on the side stream meanwhile
+    // (a check every fourth step, 20k triangles: 37.8 us a step against 39.0 with the sort behind it).
+    // The particle kernel reads the sorted state before its own wait, so it has to follow a join by an event.
+    const bool sorts = sorts_at(ctx, ctx->steps_done + 1);
+    const bool side_sort = sorts && !timed;
     if (side_sort) {
         cudaEventRecord(ctx->ev_fork, ctx->stream);       // errors surface through cudaGetLastError
         cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
         do_sort(ctx, ctx->side);
         launches += 4;
         cudaEventRecord(ctx->ev_join, ctx->side);
-    }
-    if (check) {
-        charge_now(ctx, ctx->q1, ctx->q1_clean, !timed);
-        ++launches;
     }
     if (ctx->patches) {
         FieldArgs W = ctx->field;
@@ -1206,8 +1224,7 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
 // bookkeeping of the step happens during capture) and replayed.
 static int graph_step(fetdpic_ctx *ctx, int pusher, long long &launches)
 {
-    const bool sorts = ctx->p.sort_interval > 0 && ctx->nblocks > 0 &&
-                       (ctx->steps_done + 1) % ctx->p.sort_interval == 0;
+    const bool sorts = sorts_at(ctx, ctx->steps_done + 1);
     const int parity = ctx->cell == ctx->cell_a ? 0 : 1;
     const int late = ctx->p.precision == FETDPIC_FP32 && late_step(ctx, kernels_of(ctx, pusher)) ? 1 : 0;
     const int fields = ctx->e == ctx->e_a ? 0 : 1;
@@ -1231,11 +1248,7 @@ static int graph_step(fetdpic_ctx *ctx, int pusher, long long &launches)
     // host-side effects of the step the graph replays
     ++ctx->steps_done;
     ctx->q_prev_valid = false;
-    if (sorts) {
-        std::swap(ctx->cell, ctx->cell_tmp);
-        std::swap(ctx->id, ctx->id_tmp);
-        for (int k = 0; k < 4; ++k) std::swap(ctx->f[k], ctx->f_tmp[k]);
-    }
+    if (sorts) swap_particles(ctx);
     return FETDPIC_OK;
 }
 
@@ -1272,9 +1285,7 @@ static int cycle_step(fetdpic_ctx *ctx, int pusher, long long &launches)
     if (merge && ((L - 1) & 1)) swap_fields(ctx);
     ctx->steps_done += L;
     ctx->q_prev_valid = false;
-    std::swap(ctx->cell, ctx->cell_tmp);
-    std::swap(ctx->id, ctx->id_tmp);
-    for (int k = 0; k < 4; ++k) std::swap(ctx->f[k], ctx->f_tmp[k]);
+    if (sorts_at(ctx, ctx->steps_done)) swap_particles(ctx);
     return FETDPIC_OK;
 }
 
