@@ -102,14 +102,17 @@ typedef struct {
     int precision;           /* fetdpic_precision */
     int spai_level;          /* sparsity level k >= 1 of the SPAI of [*eps] (Sec. II.A); 0 = 2;
                                 -1 = exact inverse (dense, only for <= 4096 free edges) */
-    int sort_interval;       /* steps between counting sorts of particles by triangle; 0 = 16, <0 = never */
+    int sort_interval;       /* steps between counting sorts of particles by triangle; 0 = 16, <0 = never
+                                (never either for up to 2,048 particle slots, species padded to 1,024) */
     int max_crossings;       /* walk limit per particle per step; 0 = 64 */
     int check_interval;      /* every k-th step also computes the continuity and Gauss-law
                                 residuals (FP64); 0 = never */
     int record_walk;         /* > 0: keep up to this many crossed edges per particle of the
                                 last step (debug / parity; costs bandwidth); 0 = off */
     int block_size;          /* particle-kernel threads per block; 0 = tuned default */
-    int use_graphs;          /* 1 = replay steps from a captured CUDA graph; 0 = plain launches */
+    int use_graphs;          /* 1 = replay whole sort cycles and single steps from captured CUDA
+                                graphs (other runs of steps are launched plainly); 0 = plain
+                                launches */
     int time_stages;         /* 1 = record CUDA events between stages (fetdpic_stage_times) */
     int kernel_variant;      /* FP32 particle kernel, one particle per thread: 2, 3 or 4 =
                                 256-thread blocks, that many resident per SM; 5 = particle state
@@ -143,8 +146,10 @@ typedef struct {
     int fuse_field_update;   /* 1 = the Ampere update (C^T [*mu^-1] b - i, then the SPAI
                                 product) runs as one cooperative launch whose blocks meet at a
                                 grid barrier with a bounded wait (FETDPIC_ETIMEOUT if it gives
-                                up); 0 = two launches (the default: measured faster on GB300).
-                                Same arithmetic, same results. */
+                                up); 0 = one launch of independent mesh patches, which inside a
+                                call carries the next step's Faraday update too, or two launches
+                                where the patches do not fit shared memory (the default: faster
+                                on GB300).  Same arithmetic, same results. */
 } fetdpic_params;
 
 /* One simulation instance (mesh + fields).  Instances share nothing but the

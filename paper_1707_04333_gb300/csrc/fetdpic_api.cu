@@ -218,8 +218,10 @@ struct fetdpic_ctx {
 };
 
 // Reads of up to this many bytes go through the context's page-locked buffer (one copy and one wait:
-// a particle read took three pageable copies, each a wait of its own, and a fourth for the status).
-constexpr size_t SMALL_READ = 64 * 1024;
+// a particle read took three pageable copies, each a wait of its own, and a fourth for the status).  A
+// field read of 160 KB takes 37 us so against 55 in pageable copies, of 315 KB 49 against 61; of 640 KB, 78
+// against 68: there the host's own copy out of the buffer costs more than the waits.
+constexpr size_t SMALL_READ = 384 * 1024;
 
 #define CK(call)                                                                     \
     do {                                                                             \
@@ -426,9 +428,12 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
     ctx->nfree = (long long)mrow.size();
     const bool f32 = P.precision == FETDPIC_FP32;
     // the field update by patches, unless the cooperative form is asked for or a patch's edges do
-    // not fit its block (a dense inverse)
+    // not fit its block (a dense inverse).  Beyond PATCH_MAX_F triangles the update is bound by memory
+    // bandwidth, of which the three kernels need less (us a step: 0.72 M triangles 95.9 by patches, 99.6
+    // without; 2 M 251 and 259; 3.4 M 451 and 449, in 64 instances with 18.8 M particles 622 and 610).
+    constexpr int PATCH_MAX_F = 2500000;
     PatchSet ps;
-    if (!P.fuse_field_update && P.spai_level >= 0) {
+    if (!P.fuse_field_update && P.spai_level >= 0 && ctx->F <= PATCH_MAX_F) {
         std::vector<int> te(3 * (size_t)ctx->F), row(ctx->E, -1);
         for (int f = 0; f < ctx->F; ++f)
             for (int m = 0; m < 3; ++m) te[3 * (size_t)f + m] = tp[f].ew[m] >> 1;
@@ -1504,12 +1509,13 @@ extern "C" int fetdpic_read(fetdpic_ctx *ctx, int inst, double *e, double *b, do
     const HostMesh &M = ctx->mesh[inst];
     CK(cudaSetDevice(ctx->device));
     {
-        // to the caller's edge and triangle order on the device, then to the host
+        // to the caller's edge and triangle order on the device (in one launch: 2,000 to 30,000 triangles
+        // 12-14 us less than with one for each array), then to the host
         const int eo = ctx->edge_off[inst], co = ctx->cell_off[inst];
         double *oe = ctx->field_out, *oj = oe + M.ne, *ob = oj + M.ne;
-        if (e) launch_gather_field(ctx->stream, M.ne, eo, ctx->edge_c2i, ctx->e, oe);
-        if (b) launch_gather_field(ctx->stream, M.nf, co, ctx->tri_c2i, ctx->b, ob);
-        if (j) launch_gather_field(ctx->stream, M.ne, eo, ctx->edge_c2i, ctx->j, oj);
+        if (e || b || j)
+            launch_gather_fields(ctx->stream, GatherFields{M.ne, M.nf, eo, co, ctx->edge_c2i, ctx->tri_c2i, e ? ctx->e : nullptr,
+                                                           j ? ctx->j : nullptr, b ? ctx->b : nullptr, oe});
         CK(cudaGetLastError());
         const size_t be = sizeof(double) * M.ne, bf = sizeof(double) * M.nf;
         if ((e || b || j) && 2 * be + bf <= SMALL_READ) {

@@ -286,7 +286,7 @@ struct AmpereArgs {
     const double *inst_unit;                  // (q_ref/dt) 2^-shift per instance
     const double *inst_dt;
     const double *b;
-    unsigned long long *ifix;                 // read and cleared
+    unsigned long long *ifix;                 // read; the next Faraday clears it
     double *r, *d, *j;
     float *r32;                               // FP32 copy of r (FP32 path), or null
     long long nfree;
@@ -393,8 +393,14 @@ void launch_ingest(cudaStream_t st, long long n, long long cap, long long off, i
 // *dst = v, in stream order.
 void launch_set_value(cudaStream_t st, double *dst, double v);
 
-// dst[k] = src[off + c2i[off + k]]: one instance's edge or triangle values in the caller's order.
-void launch_gather_field(cudaStream_t st, int n, int off, const int *c2i, const double *src, double *dst);
+// One instance's e, j and b (NULL: not asked for) in the caller's order, behind one another in out: ne, ne, nf values.
+struct GatherFields {
+    int ne, nf, eo, fo;                       // edges, triangles, their offsets
+    const int *edge_c2i, *tri_c2i;
+    const double *e, *j, *b;
+    double *out;
+};
+void launch_gather_fields(cudaStream_t st, const GatherFields &a);
 
 void launch_unsort64(cudaStream_t st, long long n, const int *cell, const int *id, const double *x,
                      const double *y, const double *ux, const double *uy, long long off, long long cap,

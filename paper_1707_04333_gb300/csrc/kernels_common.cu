@@ -453,16 +453,21 @@ void launch_ingest(cudaStream_t st, long long n, long long cap, long long off, i
 __global__ void k_set_value(double *dst, double v) { *dst = v; }
 void launch_set_value(cudaStream_t st, double *dst, double v) { k_set_value<<<1, 1, 0, st>>>(dst, v); }
 
-__global__ void __launch_bounds__(256) k_gather_field(int n, int off, const int *__restrict__ c2i,
-                                                      const double *__restrict__ src, double *__restrict__ dst)
+__global__ void __launch_bounds__(256) k_gather_fields(GatherFields a)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) dst[k] = src[off + c2i[off + k]];
+    if (k < a.ne) {
+        const int i = a.eo + a.edge_c2i[a.eo + k];
+        if (a.e) a.out[k] = a.e[i];
+        if (a.j) a.out[a.ne + k] = a.j[i];
+    }
+    if (a.b && k < a.nf) a.out[2 * (size_t)a.ne + k] = a.b[a.fo + a.tri_c2i[a.fo + k]];
 }
 
-void launch_gather_field(cudaStream_t st, int n, int off, const int *c2i, const double *src, double *dst)
+void launch_gather_fields(cudaStream_t st, const GatherFields &a)
 {
-    if (n > 0) k_gather_field<<<(n + 255) / 256, 256, 0, st>>>(n, off, c2i, src, dst);
+    const int n = std::max(a.e || a.j ? a.ne : 0, a.b ? a.nf : 0);
+    if (n > 0) k_gather_fields<<<(n + 255) / 256, 256, 0, st>>>(a);
 }
 
 __global__ void k_unsort64(long long off, long long cap, long long n, const int *__restrict__ cell, const int *__restrict__ id,
