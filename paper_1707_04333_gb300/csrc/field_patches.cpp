@@ -108,7 +108,7 @@ PatchSet build_patches(const PatchInput &in, int T)
         for (int m = 0; m < 3; ++m) seen = std::max(seen, in.tedge[3 * f + m] + 1);
     }
     own[np] = seen;
-    const int nth = (int)std::max(1u, std::min({16u, std::thread::hardware_concurrency(), (unsigned)((np + 15) / 16)}));
+    const int nth = (int)std::max(1u, std::min({16u, std::thread::hardware_concurrency(), (unsigned)((np + 7) / 8)}));
     if (nth == 1) {
         PatchSet S;
         S.soff.assign(1, 0);
