@@ -106,6 +106,10 @@ F64I_FN bool f64_within(double a)
     const u32 h = f64_hi(a) & 0x7fffffffu;
     return h - ((1023u - LO) << 20) < ((u32)(LO + HI) << 20) || (h | f64_lo(a)) == 0u;
 }
+F64I_FN bool f64_positive(double a)           // normal and above zero
+{
+    return f64_hi(a) - 0x100000u < 0x7fe00000u;
+}
 F64I_FN bool is_neg(double a)                 // a < 0 (not for NaN)
 {
     const u32 h = f64_hi(a);

@@ -113,7 +113,10 @@ __device__ __forceinline__ double gam2(double ux, double uy, double ic2)
     return A::root(1.0 + A::mul(A::mul(ux, ux) + A::mul(uy, uy), ic2));
 }
 
-// `ok` (integer form): cleared when u' or u^- leaves the range the rest is safe for.
+// `ok` (integer form): cleared when u' or u^- leaves the range the rest is safe for, and where the
+// gamma of the quartic is the root of exactly 0: sigma + sqrt(sigma^2 + 4 beta^2) cancels completely from
+// |beta| of about 2^27 on, and sqrt_i takes positive numbers only.  (The FP64 instructions then find
+// beta / 0 and report the particle as not finite.)
 template <class A, int PUSHER>
 __device__ __forceinline__ Push push64(double ux, double uy, double Ex, double Ey, double Bz,
                                        double alpha, double ic2, bool &ok)
@@ -133,7 +136,9 @@ __device__ __forceinline__ Push push64(double ux, double uy, double Ex, double E
         if (A::SOFT) ok = ok && f64_within<120, 64>(upx) && f64_within<120, 64>(upy);
         const double gp = gam2<A>(upx, upy, ic2);
         const double sigma = A::mul(gp, gp) - bb;
-        const double gn = A::root(A::half(sigma + A::root(A::mul(sigma, sigma) + A::four(bb))));
+        const double gn2 = A::half(sigma + A::root(A::mul(sigma, sigma) + A::four(bb)));
+        if (A::SOFT) ok = ok && f64_positive(gn2);
+        const double gn = A::root(gn2);
         const double tz = A::div(bz, gn);
         const double s = A::div(1.0, 1.0 + A::mul(tz, tz));
         out.ux = A::mul(s, upx + A::mul(upy, tz));
@@ -149,8 +154,9 @@ __device__ __forceinline__ Push push64(double ux, double uy, double Ex, double E
     if (PUSHER == FETDPIC_HC) {
         // Sec. II.C(c): gamma_H from sigma = gamma_B^2 - |beta|^2 (u^- . beta = 0 in 2-D TE)
         const double sigma = A::mul(gbar, gbar) - bb;
-        const double gh = A::root(A::half(sigma + A::root(A::mul(sigma, sigma) + A::four(bb))));
-        tz = A::div(bz, gh);
+        const double gh2 = A::half(sigma + A::root(A::mul(sigma, sigma) + A::four(bb)));
+        if (A::SOFT) ok = ok && f64_positive(gh2);
+        tz = A::div(bz, A::root(gh2));
     } else if (PUSHER == FETDPIC_BORIS_TAN) {
         // (sqrt(bz^2) and bz / |bz| are exact where bz^2 does not underflow)
         const double nb = A::SOFT ? fabs(bz) : sqrt(bb);
