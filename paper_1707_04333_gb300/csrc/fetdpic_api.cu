@@ -1223,6 +1223,24 @@ static long long enqueue_step(fetdpic_ctx *ctx, int pusher, bool timed, bool beg
     return launches;
 }
 
+// Ends the capture begun on the context stream and makes `g` of it.  A launch refused meanwhile is not
+// in the graph: then nothing is kept, and the error is reported.
+static int end_capture(fetdpic_ctx *ctx, cudaGraphExec_t &g)
+{
+    cudaGraph_t graph = nullptr;
+    const cudaError_t refused = cudaGetLastError();
+    cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
+    if (e != cudaSuccess) return ctx->cuda_fail(e, "cudaStreamEndCapture");
+    e = refused;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&g, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {
+        g = nullptr;
+        return ctx->cuda_fail(e, refused != cudaSuccess ? "launch during capture" : "cudaGraphInstantiate");
+    }
+    return FETDPIC_OK;
+}
+
 // One step through a captured graph: the launch sequence of a step depends only
 // on the pusher, which particle buffer is current and whether the step sorts,
 // so each combination is captured once (capture enqueues nothing; the host-side
@@ -1235,14 +1253,14 @@ static int graph_step(fetdpic_ctx *ctx, int pusher, long long &launches)
     const int fields = ctx->e == ctx->e_a ? 0 : 1;
     cudaGraphExec_t &g = ctx->graph[pusher][parity][sorts ? 1 : 0][late][fields];
     if (!g) {
-        cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
         const long long n = enqueue_step(ctx, pusher, false);
-        cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
-        if (e != cudaSuccess) return ctx->cuda_fail(e, "cudaStreamEndCapture");
-        e = cudaGraphInstantiate(&g, graph, 0);
-        cudaGraphDestroy(graph);
-        if (e != cudaSuccess) { g = nullptr; return ctx->cuda_fail(e, "cudaGraphInstantiate"); }
+        const int rc = end_capture(ctx, g);
+        if (rc) {                                 // no step was taken
+            --ctx->steps_done;
+            if (sorts) swap_particles(ctx);
+            return rc;
+        }
         ctx->graph_launches[pusher][parity][sorts ? 1 : 0][late][fields] = n;
         CK(cudaGraphLaunch(g, ctx->stream));
         launches += n;
@@ -1270,15 +1288,16 @@ static int cycle_step(fetdpic_ctx *ctx, int pusher, long long &launches)
     const bool merge = can_merge(ctx, L - 1);
     cudaGraphExec_t &g = ctx->cycle[pusher][parity][fields];
     if (!g) {
-        cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
         long long n = 0;
         for (int k = 0; k < L; ++k) n += enqueue_step(ctx, pusher, false, merge && k > 0, merge && k + 1 < L);
-        cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
-        if (e != cudaSuccess) return ctx->cuda_fail(e, "cudaStreamEndCapture");
-        e = cudaGraphInstantiate(&g, graph, 0);
-        cudaGraphDestroy(graph);
-        if (e != cudaSuccess) { g = nullptr; return ctx->cuda_fail(e, "cudaGraphInstantiate"); }
+        const int rc = end_capture(ctx, g);
+        if (rc) {                                 // no step was taken
+            if (merge && ((L - 1) & 1)) swap_fields(ctx);
+            if (sorts_at(ctx, ctx->steps_done)) swap_particles(ctx);
+            ctx->steps_done -= L;
+            return rc;
+        }
         ctx->cycle_launches[pusher][parity][fields] = n;
         CK(cudaGraphLaunch(g, ctx->stream));
         launches += n;

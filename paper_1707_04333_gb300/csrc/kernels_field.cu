@@ -184,12 +184,14 @@ __global__ void __launch_bounds__(NT, NT == NT_LARGE ? PER_SM : 4) k_field(Field
     }
 }
 
+// The limit belongs to the kernel, for every context of the process: always the same value, since one
+// context's smaller need would take from another's.
 template <typename V, int FAR, bool EXT>
-cudaError_t setup(size_t smem)
+cudaError_t setup()
 {
-    cudaError_t e = cudaFuncSetAttribute(k_field<V, FAR, EXT, NT_SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_field<V, FAR, EXT, NT_LARGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr cudaFuncAttribute limit = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_field<V, FAR, EXT, NT_SMALL>, limit, (int)FIELD_SMEM_MAX);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_field<V, FAR, EXT, NT_LARGE>, limit, (int)FIELD_SMEM_MAX);
     return e;
 }
 
@@ -226,11 +228,11 @@ size_t field_smem(bool f32, int max_r, int max_e)
 cudaError_t field_setup(size_t smem)
 {
     if (smem <= 48 * 1024) return cudaSuccess;         // what every kernel may use
-    cudaError_t e = setup<float, 0, false>(smem);
-    if (e == cudaSuccess) e = setup<float, 1, false>(smem);
-    if (e == cudaSuccess) e = setup<float, 1, true>(smem);
-    if (e == cudaSuccess) e = setup<double, 0, false>(smem);
-    if (e == cudaSuccess) e = setup<double, 2, false>(smem);
+    cudaError_t e = setup<float, 0, false>();
+    if (e == cudaSuccess) e = setup<float, 1, false>();
+    if (e == cudaSuccess) e = setup<float, 1, true>();
+    if (e == cudaSuccess) e = setup<double, 0, false>();
+    if (e == cudaSuccess) e = setup<double, 2, false>();
     return e;
 }
 
