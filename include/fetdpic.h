@@ -87,9 +87,11 @@ typedef enum {
      * positions and momenta (Boris-tan excepted: tan is not correctly rounded). */
     FETDPIC_FP64 = 0,
     /* FP32 gather/push/deposit with cell-local barycentric positions and
-     * momenta in units of c; double-float (48 bits; FP64 beyond its range) for
-     * the Lorentz factor and momentum update of particles with gamma > 10;
-     * FP64 for the field unknowns e, b, the Faraday update, C^T [*mu^-1] b - i
+     * momenta in units of c; for particles with gamma > 10 the Lorentz factor
+     * and momentum update in two and three floats, whose error against
+     * extended precision is below that of the same push in FP64 with Newton
+     * roots, or in FP64 (gamma above 3.1e8; a kick or |q B dt / 2m| above
+     * gamma / 8, gamma / 31 for Boris-tan); FP64 for the field unknowns e, b, the Faraday update, C^T [*mu^-1] b - i
      * and the checks.  The SPAI product dt M r of
      * the Ampere update runs in FP32 (FP32 matrix values, r rounded to FP32,
      * FP32 sums) and is added to the FP64 e. */

@@ -12,6 +12,7 @@
 
 #include <cuda_runtime.h>
 
+#include "double_float.h"
 #include "fetdpic_internal.h"
 #include "field_device.cuh"
 
@@ -146,192 +147,16 @@ __device__ __forceinline__ T push_c1(T &ux, T &uy, T ex, T ey, T bz)
     return rsq<T, NEWTON>(one + ux * ux + uy * uy);
 }
 
-// ------------------------------------------------- double-float arithmetic
-// A value held as an unevaluated sum h + l of two floats, |l| of a few ulp(h) at
-// most: some 47 significand bits from FP32 additions and fused multiply-adds
-// (Dekker 1971; Knuth's two-sum).  GB300 issues FP32 at 128 lanes per SM and
-// clock and FP64 at 2, so the operations of one double-float operation take a
-// fraction of one FP64 instruction's time.  The rounding intrinsics keep the
-// error terms from being contracted.  A result is renormalised only where it is
-// used as a single float: products and sums take a low part of a few ulp as well
-// as one of half an ulp.
-struct F2 {
-    float h, l;
-    __device__ __forceinline__ F2() {}
-    __device__ __forceinline__ F2(float a, float b) : h(a), l(b) {}
-};
-__device__ __forceinline__ F2 quick_two_sum(float a, float b)          // |a| >= |b|
-{
-    const float s = __fadd_rn(a, b);
-    return F2(s, __fsub_rn(b, __fsub_rn(s, a)));
-}
-__device__ __forceinline__ F2 two_sum(float a, float b)
-{
-    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-    return F2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t)));
-}
-__device__ __forceinline__ F2 two_prod(float a, float b)
-{
-    const float p = __fmul_rn(a, b);
-    return F2(p, __fmaf_rn(a, b, -p));
-}
-__device__ __forceinline__ F2 add_small(const F2 &a, float b)          // |a| >= |b|
-{
-    const F2 s = quick_two_sum(a.h, b);
-    return F2(s.h, __fadd_rn(s.l, a.l));
-}
-__device__ __forceinline__ F2 add_small(const F2 &a, const F2 &b)
-{
-    const F2 s = quick_two_sum(a.h, b.h);
-    return F2(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ F2 operator*(const F2 &a, const F2 &b)
-{
-    const F2 p = two_prod(a.h, b.h);
-    return F2(p.h, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, p.l)));
-}
-__device__ __forceinline__ F2 operator*(const F2 &a, float b)
-{
-    const F2 p = two_prod(a.h, b);
-    return F2(p.h, __fmaf_rn(a.l, b, p.l));
-}
-__device__ __forceinline__ F2 sqr(const F2 &a)
-{
-    const F2 p = two_prod(a.h, a.h);
-    return F2(p.h, __fmaf_rn(__fadd_rn(a.h, a.h), a.l, p.l));
-}
-__device__ __forceinline__ F2 scale(const F2 &a, float p2) { return F2(a.h * p2, a.l * p2); }   // p2: a power of two
-// 1/sqrt(x), sqrt(x), 1/x: a single-precision seed and one Newton-Raphson step
-// whose residual 1 - x y^2 (1 - x y) is formed without rounding its leading
-// part; relative error about 1e-13, as that of the step in FP64 (the seed's
-// error squared).
-__device__ __forceinline__ float rsqrt_residual(const F2 &x, float y, F2 &xy)
-{
-    xy = two_prod(x.h, y);
-    xy.l = __fmaf_rn(x.l, y, xy.l);
-    return __fmaf_rn(-xy.l, y, __fmaf_rn(-xy.h, y, 1.f));
-}
-__device__ __forceinline__ F2 rsqrt_f2(const F2 &x)
-{
-    const float y = rsqrtf(x.h);
-    F2 xy;
-    return F2(y, 0.5f * y * rsqrt_residual(x, y, xy));
-}
-__device__ __forceinline__ F2 sqrt_f2(const F2 &x)
-{
-    const float y = rsqrtf(x.h);
-    F2 xy;
-    const float e = rsqrt_residual(x, y, xy);
-    return F2(xy.h, __fmaf_rn(0.5f * xy.h, e, xy.l));
-}
-__device__ __forceinline__ F2 rcp_f2(const F2 &x)
-{
-    const float y = __fdividef(1.f, x.h);
-    return F2(y, y * __fmaf_rn(-x.l, y, __fmaf_rn(-x.h, y, 1.f)));
-}
-
-// Both components of a vector in one register pair: the packed FP32 instructions
-// round each half as the scalar ones do and take one issue slot for two
-// operations (the rate in lanes is the same: 120 per SM and clock either way),
-// and it is issue slots that a kernel full of pushes is bound by (71 % of them
-// used, FP32 pipe 43 %).  Packed, and renormalised only at the end: 6.25 M
-// particles above gamma = 10 took 183.7 us a step before, 154.9 after
-// (Higuera-Cary; Vay 189.4 and 160.4, Boris 169.4 and 147.2, Boris-tan 234.7
-// and 216.4).  Against extended precision over gamma 10 to 3e8, kick and |beta|
-// up to gamma / 8, u stays within 7e-14 and 1/gamma within 1.3e-13 of their size
-// before the rounding to FP32, whose 6e-8 is all that the stored values show.
-struct V2 { unsigned long long v; };
-__device__ __forceinline__ V2 vec(float x, float y)
-{
-    V2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ void parts(V2 a, float &x, float &y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v)); }
-__device__ __forceinline__ V2 operator+(V2 a, V2 b)
-{
-    V2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ V2 operator-(V2 a, V2 b)
-{
-    V2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ V2 operator*(V2 a, V2 b)
-{
-    V2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ V2 fma(V2 a, V2 b, V2 c)
-{
-    V2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
-__device__ __forceinline__ V2 neg(V2 a)
-{
-    float x, y;
-    parts(a, x, y);
-    return vec(-x, -y);
-}
-__device__ __forceinline__ V2 swap(V2 a)
-{
-    float x, y;
-    parts(a, x, y);
-    return vec(y, x);
-}
-struct D2 { V2 h, l; };                                                // a vector of two double-floats
-__device__ __forceinline__ D2 two_sum(V2 a, V2 b)
-{
-    const V2 s = a + b, t = s - a;
-    return D2{s, (a - (s - t)) + (b - t)};
-}
-__device__ __forceinline__ D2 normal(const D2 &a)
-{
-    const V2 s = a.h + a.l;
-    return D2{s, a.l - (s - a.h)};
-}
-__device__ __forceinline__ D2 operator*(const D2 &a, const D2 &b)
-{
-    const V2 p = a.h * b.h;
-    return D2{p, fma(a.l, b.h, fma(a.h, b.l, fma(a.h, b.h, neg(p))))};
-}
-__device__ __forceinline__ D2 operator+(const D2 &a, const D2 &b)
-{
-    const D2 s = two_sum(a.h, b.h);
-    return D2{s.h, s.l + (a.l + b.l)};
-}
-__device__ __forceinline__ D2 operator+(const D2 &a, V2 b)
-{
-    const D2 s = two_sum(a.h, b);
-    return D2{s.h, s.l + a.l};
-}
-// (a_y, a_x) (s, -s)
-__device__ __forceinline__ D2 cross(const D2 &a, const F2 &s)
-{
-    return D2{swap(a.h), swap(a.l)} * D2{vec(s.h, -s.h), vec(s.l, -s.l)};
-}
-__device__ __forceinline__ D2 operator*(const D2 &a, const F2 &s) { return a * D2{vec(s.h, s.h), vec(s.l, s.l)}; }
-// 1 + a_x^2 + a_y^2, where |a| > 1
-__device__ __forceinline__ F2 one_plus_norm2(const D2 &a)
-{
-    const V2 p = a.h * a.h, l = fma(a.h + a.h, a.l, fma(a.h, a.h, neg(p)));
-    float px, py, lx, ly;
-    parts(p, px, py);
-    parts(l, lx, ly);
-    const F2 s = two_sum(px, py);
-    return add_small(F2(s.h, __fadd_rn(s.l, __fadd_rn(lx, ly))), 1.f);
-}
-
-// The push for gamma > 10, where FP32 loses 1 - v/c and the cancellation in
-// sigma: the formulas of push_c1 in double-float (rare in thermal plasmas,
-// every particle of a high-gamma beam; kept out of line so its registers do
-// not count against the FP32 main path).  Arguments and result by value, so no
-// caller variable needs an address.  Returns (u_x, u_y, v_x, v_y) in units of c.
+// The push for gamma > 10: the formulas of push_c1 in double-float (rare in
+// thermal plasmas, every particle of a high-gamma beam; kept out of line so its
+// registers do not count against the FP32 main path).  Arguments and result by
+// value, so no caller variable needs an address.  Returns (u_x, u_y, v_x, v_y)
+// in units of c.
+//
+// 6.25 M particles above gamma = 10, us a step with the push in FP64 and here:
+// Higuera-Cary 707 and 162, Vay 705 and 165, Boris 565 and 153, Boris-tan 989
+// and 219.  Without the third floats and the roots' second term, 47 bits
+// throughout and an error above the FP64 push's, it took 155, 161, 147 and 215.
 struct PushOut { float ux, uy, vx, vy; };
 
 // The same in FP64, for what double-float cannot hold.
@@ -359,49 +184,10 @@ __device__ __forceinline__ bool f2_takes(float g2, float ex, float ey, float bz)
 template <int PUSHER>
 __device__ __noinline__ PushOut push_f2(float ux, float uy, float ex, float ey, float bz)
 {
-    // gamma > 10, |kick| < gamma / 8 and |beta| < gamma / 8, so |u^-|^2, |u'|^2 and |u^{n+1}|^2 exceed
-    // both 1 and |beta|^2, and t^2 < 1: those sums need no two-sum
-    const V2 u = vec(ux, uy), eps = vec(ex, ey);
-    D2 x;                                                              // u^{n+1/2}
-    F2 ig;                                                             // 1/gamma^{n+1/2}
-    if (PUSHER == FETDPIC_VAY) {
-        const F2 w = rsqrt_f2(one_plus_norm2(D2{u, V2{0ull}})) * bz;
-        const D2 up = normal(cross(D2{u, V2{0ull}}, w) + (two_sum(u, eps) + eps));
-        const F2 bb = two_prod(bz, bz);
-        const F2 sigma = add_small(one_plus_norm2(up), F2(-bb.h, -bb.l));
-        const F2 root = sqrt_f2(add_small(sqr(sigma), scale(bb, 4.f)));
-        ig = rsqrt_f2(scale(add_small(root, sigma), 0.5f));
-        const F2 tz = ig * bz, q = sqr(tz);
-        const F2 s = rcp_f2(add_small(F2(1.f, 0.f), q));
-        x = normal((up + cross(up, tz)) * s);
-    } else {
-        const D2 um = two_sum(u, eps);                                 // u^-
-        const F2 g2 = one_plus_norm2(um);
-        F2 tz;
-        if (PUSHER == FETDPIC_HC) {
-            const F2 bb = two_prod(bz, bz);
-            const F2 sigma = add_small(g2, F2(-bb.h, -bb.l));
-            const F2 root = sqrt_f2(add_small(sqr(sigma), scale(bb, 4.f)));
-            tz = rsqrt_f2(scale(add_small(root, sigma), 0.5f)) * bz;
-        } else {
-            tz = rsqrt_f2(g2) * bz;
-            if (PUSHER == FETDPIC_BORIS_TAN) {
-                // tan t = t + t (t^2/3 + 2 t^4/15 + 17 t^6/315 + 62 t^8/2835 + ...): the first
-                // neglected term is below 1e-15 of t for |t| < 0.04
-                const F2 q = sqr(tz);
-                const float r = q.h * q.h * (2.f / 15.f + q.h * (17.f / 315.f + q.h * (62.f / 2835.f)));
-                // 1/3 as a double-float: 1/3 rounded to FP32, and the rest
-                const float third = 1.f / 3.f, rest = (float)(1.0 / 3.0 - (double)third);
-                tz = add_small(tz, tz * add_small(q * F2(third, rest), r));
-            }
-        }
-        const F2 sz = scale(tz, 2.f) * rcp_f2(add_small(F2(1.f, 0.f), sqr(tz)));
-        x = normal(um + cross(um + cross(um, tz), sz) + eps);
-        ig = rsqrt_f2(one_plus_norm2(x));
-    }
-    const D2 v = normal(x * ig);
+    const HighPush p = high_gamma_push<PUSHER>(ux, uy, ex, ey, bz);
+    const D2 v = normal(p.u.x * normal(p.ig));
     PushOut o;
-    parts(x.h, o.ux, o.uy);
+    parts(p.u.x.h, o.ux, o.uy);
     parts(v.h, o.vx, o.vy);
     return o;
 }
