@@ -257,12 +257,12 @@ static int take_status(fetdpic_ctx *ctx)
     CK(cudaMemcpyAsync(st, ctx->status, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     const unsigned s = *st;
-    if (s) CK(cudaMemset(ctx->status, 0, sizeof(unsigned)));
+    if (s) CK(cudaMemsetAsync(ctx->status, 0, sizeof(unsigned), ctx->stream));
     // a step that timed out is incomplete: drop the current it deposited, and the counts a grid
     // barrier that gave up left behind
     if (s & ST_TIMEOUT) {
-        if (ctx->gbar) CK(cudaMemset(ctx->gbar, 0, sizeof(unsigned) * GBAR_WORDS));
-        if (ctx->ifix) CK(cudaMemset(ctx->ifix, 0, sizeof(unsigned long long) * ctx->E));
+        if (ctx->gbar) CK(cudaMemsetAsync(ctx->gbar, 0, sizeof(unsigned) * GBAR_WORDS, ctx->stream));
+        if (ctx->ifix) CK(cudaMemsetAsync(ctx->ifix, 0, sizeof(unsigned long long) * ctx->E, ctx->stream));
     }
     return map_status(ctx, s);
 }
@@ -584,16 +584,16 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
             ctx->m_row = ctx->alloc<int>(mrow.size());
             ctx->m_ci = ctx->alloc<int>(sci.size());
             ctx->r = ctx->alloc<double>(ctx->E);
-            CK(cudaMemset(ctx->r, 0, sizeof(double) * ctx->E));
+            CK(cudaMemsetAsync(ctx->r, 0, sizeof(double) * ctx->E, ctx->stream));
             if (f32) {
                 ctx->r32 = ctx->alloc<float>(ctx->E);
-                CK(cudaMemset(ctx->r32, 0, sizeof(float) * ctx->E));     // read by the SPAI product
+                CK(cudaMemsetAsync(ctx->r32, 0, sizeof(float) * ctx->E, ctx->stream));     // read by the SPAI product
             }
         }
         ctx->e_a = ctx->e;
         ctx->status = ctx->alloc<unsigned>(1);
         ctx->gbar = ctx->alloc<unsigned>(GBAR_WORDS);
-        if (ctx->gbar) CK(cudaMemset(ctx->gbar, 0, sizeof(unsigned) * GBAR_WORDS));
+        if (ctx->gbar) CK(cudaMemsetAsync(ctx->gbar, 0, sizeof(unsigned) * GBAR_WORDS, ctx->stream));
         if (P.check_interval > 0) {
             ctx->nrp = ctx->alloc<int>(nrp.size());
             ctx->nedge = ctx->alloc<int>(nedge.size());
@@ -1714,7 +1714,7 @@ extern "C" int fetdpic_check(fetdpic_ctx *ctx, int inst, double *dce_max, double
     if (dce_max) *dce_max = v[0];
     if (dgl_max) *dgl_max = v[1];
     if (energy) *energy = v[2];
-    CK(cudaMemset(ctx->chk_out + 3 * inst, 0, 2 * sizeof(double)));   // maxima restart; energy stays
+    CK(cudaMemsetAsync(ctx->chk_out + 3 * inst, 0, 2 * sizeof(double), ctx->stream));   // maxima restart; energy stays
     return take_status(ctx);
 }
 
