@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(FUSED_BLOCK) k_ampere_fused(AmpereArgs a)
 template <typename V>
 static void launch_fused(cudaStream_t st, const AmpereArgs &a)
 {
-    static int per_sm = 0, sms = 0, dev = -1;
+    static thread_local int per_sm = 0, sms = 0, dev = -1;
     int d = 0;
     cudaGetDevice(&d);
     if (d != dev || per_sm == 0) {
@@ -360,10 +360,10 @@ __global__ void __launch_bounds__(256) k_scatter(long long nchunks, const int *_
     }
 }
 
-// SM count of the current device (cached per device).
+// SM count of the current device (each thread keeps its own: contexts step on several).
 static int sort_sms()
 {
-    static int sms = 0, dev = -1;
+    static thread_local int sms = 0, dev = -1;
     int d = 0;
     cudaGetDevice(&d);
     if (d != dev || sms == 0) { cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d); dev = d; }

@@ -953,11 +953,12 @@ __global__ void __launch_bounds__(P32_BLOCK, 3) k_particles32_staged(StepArgs32 
 
 // Persistent grid: resident blocks per SM (from the occupancy calculator) times
 // the SM count, capped by the work.  MINB = minimum resident blocks per SM the
-// register allocation targets (2, 3 or 4 x 256 threads); chosen by `variant`.
+// register allocation targets (2, 3 or 4 x 256 threads); chosen by `variant`.  What the calculator says is
+// kept per thread: contexts may step on several at once.
 template <int PUSHER, int MINB, int NW = P32_WARPS>
 static void launch_p32(cudaStream_t st, const StepArgs32 &a)
 {
-    static int per_sm = 0, sms = 0, dev = -1;
+    static thread_local int per_sm = 0, sms = 0, dev = -1;
     int d = 0;
     cudaGetDevice(&d);
     if (d != dev || per_sm == 0) {
@@ -975,7 +976,7 @@ static void launch_p32(cudaStream_t st, const StepArgs32 &a)
 template <int PUSHER, int MINB, int NW, bool SEQ = false, int WT = 0>
 static void launch_p32x2(cudaStream_t st, const StepArgs32 &a)
 {
-    static int per_sm = 0, sms = 0, dev = -1;
+    static thread_local int per_sm = 0, sms = 0, dev = -1;
     int d = 0;
     cudaGetDevice(&d);
     if (d != dev || per_sm == 0) {
@@ -993,7 +994,7 @@ static void launch_p32x2(cudaStream_t st, const StepArgs32 &a)
 template <int PUSHER>
 static void launch_p32s(cudaStream_t st, const StepArgs32 &a)
 {
-    static int per_sm = 0, sms = 0, dev = -1;
+    static thread_local int per_sm = 0, sms = 0, dev = -1;
     int d = 0;
     cudaGetDevice(&d);
     if (d != dev || per_sm == 0) {

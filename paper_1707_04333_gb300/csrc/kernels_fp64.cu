@@ -542,7 +542,8 @@ __global__ void __launch_bounds__(256, 2) k_particles64(StepArgs64 a)
 template <int PUSHER>
 static void launch_p64(cudaStream_t st, const StepArgs64 &a)
 {
-    static int per_sm = 0, sms = 0, dev = -1, blk = 0;
+    // each thread keeps its own: contexts of different block sizes may step on several at once
+    static thread_local int per_sm = 0, sms = 0, dev = -1, blk = 0;
     const size_t ring = (size_t)(a.block / 32) * RING64 * sizeof(Walk64);
     int d = 0;
     cudaGetDevice(&d);
