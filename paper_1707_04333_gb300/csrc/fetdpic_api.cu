@@ -1329,6 +1329,10 @@ extern "C" int fetdpic_step(fetdpic_ctx *ctx, long long nsteps, int pusher)
     const bool timed = ctx->p.time_stages != 0;
     const bool graphs = ctx->p.use_graphs != 0 && !timed && ctx->p.check_interval <= 0;
     const int L = ctx->p.sort_interval;
+    // a graph of the caller's own is replayed on the buffers it was captured on: there the fields stay in theirs
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(ctx->stream, &cap));
+    const bool in_place = cap != cudaStreamCaptureStatusNone;
     for (long long s = 0; s < nsteps;) {
         long long run = nsteps - s;              // steps up to the next whole cycle, or the rest
         if (graphs) {
@@ -1355,7 +1359,7 @@ extern "C" int fetdpic_step(fetdpic_ctx *ctx, long long nsteps, int pusher)
                 CK(cudaStreamSynchronize(ctx->stream));
                 collect_events(ctx);
             }
-            const bool more = can_merge(ctx, run - 1 - k);
+            const bool more = !in_place && can_merge(ctx, run - 1 - k);
             launches += enqueue_step(ctx, pusher, timed, begun, more);
             begun = more;
         }
