@@ -1768,6 +1768,11 @@ extern "C" int fetdpic_set_external_amplitude(fetdpic_ctx *ctx, int inst, double
     if (!ctx || inst < 0 || inst >= (int)ctx->mesh.size()) return FETDPIC_EINVAL;
     if (!std::isfinite(amplitude)) return ctx->fail(FETDPIC_EINVAL, "non-finite amplitude");
     CK(cudaSetDevice(ctx->device));
+    // a captured launch would set this amplitude again at every replay
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(ctx->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone)
+        return ctx->fail(FETDPIC_ECUDA, "fetdpic_set_external_amplitude: the stream is being captured");
     // stream-ordered: steps enqueued before see the old value, later ones the new
     launch_set_value(ctx->stream, ctx->ext_amp + inst, amplitude);
     CK(cudaGetLastError());
