@@ -1563,17 +1563,22 @@ extern "C" int fetdpic_read(fetdpic_ctx *ctx, int inst, double *e, double *b, do
         }
     }
     if (x || u || cell) {
+        // an error below does not return before the field copies have reached the caller's memory
         int rc = finalize(ctx);
-        if (rc) return rc;
-        if (species < 0 || species >= (int)ctx->sp.size()) {
+        if (rc == FETDPIC_OK && (species < 0 || species >= (int)ctx->sp.size()))
+            rc = ctx->fail(FETDPIC_EINVAL, "bad species");
+        if (rc) {
             CK(cudaStreamSynchronize(ctx->stream));
-            return ctx->fail(FETDPIC_EINVAL, "bad species");
+            return rc;
         }
         const Species &D = ctx->sp[species];
         if (D.n > 0) {
             const size_t bx = sizeof(double) * 2 * D.n, bc = sizeof(int) * D.n;
             char *st = (char *)xfer_buf(ctx, 2 * bx + bc);
-            if (!st) return FETDPIC_ENOMEM;
+            if (!st) {
+                CK(cudaStreamSynchronize(ctx->stream));
+                return FETDPIC_ENOMEM;
+            }
             double *ox = (double *)st, *ou = (double *)(st + bx);
             int *oc = (int *)(st + 2 * bx);
             if (ctx->p.precision == FETDPIC_FP32)
