@@ -438,8 +438,12 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         for (int f = 0; f < ctx->F; ++f)
             for (int m = 0; m < 3; ++m) te[3 * (size_t)f + m] = tp[f].ew[m] >> 1;
         for (size_t r = 0; r < mrow.size(); ++r) row[mrow[r]] = (int)r;
-        ps = build_patches(PatchInput{ctx->F, te.data(), row.data(), mrp.data(), mci.data(), mv.data()},
-                           field_patch_size(ctx->F, ctx->sms));
+        try {
+            ps = build_patches(PatchInput{ctx->F, te.data(), row.data(), mrp.data(), mci.data(), mv.data()},
+                               field_patch_size(ctx->F, ctx->sms));
+        } catch (const std::bad_alloc &) {
+            return FETDPIC_ENOMEM;
+        }
         ctx->patches = ps.ok && field_smem(f32, ps.max_r, ps.max_e) <= FIELD_SMEM_MAX;
     }
     // else sliced ELL over all rows (32 rows per slice, column-major inside a slice)

@@ -4,6 +4,7 @@
 // recomputes, and its rows of the sparse approximate inverse with columns
 // numbered inside the patch.
 #include <algorithm>
+#include <exception>
 #include <thread>
 #include <vector>
 
@@ -117,16 +118,29 @@ PatchSet build_patches(const PatchInput &in, int T)
         S.ok = np > 0 && S.max_r <= 65535;
         return S;
     }
+    // no exception leaves a thread: it is thrown again here.  A thread that cannot be started is done without
     std::vector<PatchSet> part(nth);
+    std::vector<std::exception_ptr> failed(nth);
+    auto work = [&](int t) noexcept {
+        try {
+            part[t].soff.assign(1, 0);
+            build_range(part[t], in, own, T, (int)((long long)np * t / nth), (int)((long long)np * (t + 1) / nth));
+        } catch (...) {
+            failed[t] = std::current_exception();
+        }
+    };
     {
         std::vector<std::thread> th;
-        for (int t = 0; t < nth; ++t)
-            th.emplace_back([&, t] {
-                part[t].soff.assign(1, 0);
-                build_range(part[t], in, own, T, (int)((long long)np * t / nth), (int)((long long)np * (t + 1) / nth));
-            });
+        th.reserve(nth);
+        try {
+            while ((int)th.size() < nth - 1) th.emplace_back(work, (int)th.size());
+        } catch (...) {
+        }
+        for (int t = (int)th.size(); t < nth; ++t) work(t);
         for (auto &t : th) t.join();
     }
+    for (const std::exception_ptr &e : failed)
+        if (e) std::rethrow_exception(e);
     PatchSet S;
     S.soff.assign(1, 0);
     S.T = T;
