@@ -102,6 +102,12 @@ struct PatchInput {
     const long long *mrp; const int *mci; const double *mv;
 };
 PatchSet build_patches(const PatchInput &in, int T);
+// Triangles of a patch on a mesh of F triangles.
+int field_patch_size(int F, int sms);
+// Shared memory of one block; a context whose patches need more uses launch_ampere.
+size_t field_smem(bool f32, int max_r, int max_e);
+constexpr size_t FIELD_SMEM_MAX = 100 * 1024;
+constexpr int FIELD_PER_SM = 3;             // blocks of a large patch that share an SM
 
 // Same barycentric evaluation the kernels use (gradient form, no FMA).
 void host_lambdas(const HostMesh &M, int f, double x, double y, double *l);
@@ -324,11 +330,6 @@ struct FieldArgs {
     const CstA *csta; const CstB *cstb; const double2 *dtinv; Rec32 *rec32; float inv2c2; Ext32 ext;   // FP32
     const Geo64 *geo; const Topo *topo; Rec64 *rec64;                                                // FP64
 };
-// Triangles of a patch on a mesh of F triangles.
-int field_patch_size(int F, int sms);
-// Shared memory of one block; a context whose patches need more uses launch_ampere.
-size_t field_smem(bool f32, int max_r, int max_e);
-constexpr size_t FIELD_SMEM_MAX = 100 * 1024;
 // Prepares the kernels for `smem` bytes of shared memory (once per context).
 cudaError_t field_setup(size_t smem);
 void launch_field(cudaStream_t st, const FieldArgs &a);

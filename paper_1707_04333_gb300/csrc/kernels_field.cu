@@ -30,7 +30,7 @@ constexpr int RB = 2;                       // edges of the curl phase a thread 
 // Threads of a block: 512, three blocks per SM, for patches of more than 128
 // triangles; 256 for the small meshes, whose rows are loaded whole (seven
 // pairs at a time): only latency counts there.
-constexpr int NT_LARGE = 512, NT_SMALL = 256, PER_SM = 3;
+constexpr int NT_LARGE = 512, NT_SMALL = 256, PER_SM = FIELD_PER_SM;
 template <typename V> struct Pair;
 template <> struct Pair<float> { using type = float2; };
 template <> struct Pair<double> { using type = double2; };
@@ -204,26 +204,6 @@ void go(cudaStream_t st, const FieldArgs &a)
 }
 
 }  // namespace
-
-// All patches resident at once (a second, nearly empty wave costs as much as the
-// first: 704 triangles instead of 512 took the 320k-triangle step from 51.2 to
-// 44.5 us, 448 instead of 352 the 201k-triangle one from 137 to 129), at most
-// 704 triangles each, and at least 64: smaller ones gain nothing on 2,048
-// triangles (6.77 us a step with 48, 6.71 with 64, 6.88 with 96).
-int field_patch_size(int F, int sms)
-{
-    constexpr int most = 704, least = 64;
-    const long long slots = (long long)(sms > 0 ? sms : 1) * PER_SM;
-    const long long waves = ((long long)F + slots * most - 1) / (slots * most);
-    const long long room = slots * (waves > 0 ? waves : 1);
-    const long long T = (F + room - 1) / room;
-    return (int)(T < least ? least : T);
-}
-
-size_t field_smem(bool f32, int max_r, int max_e)
-{
-    return sizeof(double) * ((size_t)max_r + max_e) + (f32 ? sizeof(float) * (size_t)max_r : 0);
-}
 
 cudaError_t field_setup(size_t smem)
 {
