@@ -51,8 +51,8 @@ struct HostMesh {
     std::vector<int> eperm, einv;
 };
 
-// Order of the triangles along a Hilbert curve of their centroids (ties by
-// index): perm[k] = the caller's index of the k-th triangle.  Neighbours end up
+// Order of the triangles along a Hilbert curve of their centroids (ties by a
+// finer curve, then by index): perm[k] = the caller's index of the k-th triangle.  Neighbours end up
 // close in memory, so particles that have crossed into a neighbour since the
 // last sort, and the sort's scattered writes, stay within cached lines.
 std::vector<int> hilbert_order(int nn, const double *xy, int nf, const int *tri);

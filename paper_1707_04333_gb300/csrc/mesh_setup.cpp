@@ -66,6 +66,25 @@ std::vector<int> hilbert_order(int nn, const double *xy, int nf, const int *tri)
         key[f] = hilbert_index(x, y, order);
     }
     std::stable_sort(perm.begin(), perm.end(), [&](int a, int b) { return key[a] < key[b]; });
+    // triangles of one cell follow the curve on a grid 2^15 times finer: a mesh refined beyond 2^16 to 1
+    // would keep them in the caller's order, neighbours far apart
+    const int fine = 31;
+    const double fscale = span > 0 ? ((1u << fine) - 1) / span : 0.0;
+    std::vector<std::pair<unsigned long long, int>> run;
+    for (int f0 = 0; f0 < nf;) {
+        int f1 = f0 + 1;
+        while (f1 < nf && key[perm[f1]] == key[perm[f0]]) ++f1;
+        if (f1 - f0 > 1) {
+            run.clear();
+            for (int f = f0; f < f1; ++f) {
+                const int k = perm[f];
+                run.push_back({hilbert_index((unsigned)((c[2 * k] - lo[0]) * fscale), (unsigned)((c[2 * k + 1] - lo[1]) * fscale), fine), k});
+            }
+            std::sort(run.begin(), run.end());
+            for (int f = f0; f < f1; ++f) perm[f] = run[f - f0].second;
+        }
+        f0 = f1;
+    }
     return perm;
 }
 

@@ -12,15 +12,15 @@ pytestmark = pytest.mark.gpu
 def _scattered(nx, seed):
     """A fine square whose triangles, in no order, share one cell of the space-filling curve because two
     more triangles lie far away: a patch's triangles are no neighbours, so it needs many other edges."""
-    m = inputs.jittered_delaunay(nx, nx, 1e-6, 1e-6, 0.2, seed=seed)
+    m = inputs.jittered_delaunay(nx, nx, 1e-10, 1e-10, 0.2, seed=seed)
     rng = np.random.default_rng(seed)
     n = len(m.nodes)
     nodes = np.concatenate([m.nodes, np.array([[1.0, 1.0], [1.001, 1.0], [1.001, 1.001], [1.0, 1.001]])])
     tri = np.concatenate([m.triangles[rng.permutation(len(m.triangles))], [[n, n + 1, n + 2], [n, n + 2, n + 3]]]).astype(np.int32)
     mesh = inputs.Mesh(nodes, tri, m.lx, m.ly)
-    x = rng.uniform(2e-7, 8e-7, (500, 2))
+    x = rng.uniform(2e-11, 8e-11, (500, 2))
     u = rng.normal(0, 0.3 * inputs.C_LIGHT, (500, 2))
-    h = 1e-6 / nx
+    h = 1e-10 / nx
     s = inputs.Species(-1e-18, 1e-18 * inputs.M_E / inputs.Q_E, x, u, np.full(500, -1, np.int32))
     return inputs.Workload("scattered", mesh, [s], 0.02 * h / inputs.C_LIGHT, b0=0.01)
 
