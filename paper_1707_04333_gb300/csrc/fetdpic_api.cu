@@ -427,8 +427,8 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         }
     ctx->nfree = (long long)mrow.size();
     const bool f32 = P.precision == FETDPIC_FP32;
-    // the field update by patches, unless the cooperative form is asked for or a patch's edges do
-    // not fit its block (a dense inverse).  Beyond PATCH_MAX_F triangles the update is bound by memory
+    // the field update by patches, unless the cooperative form is asked for, a patch's edges do not fit
+    // its block (a dense inverse) or the patches would compute too much twice.  Beyond PATCH_MAX_F triangles the update is bound by memory
     // bandwidth, of which the three kernels need less (us a step: 0.72 M triangles 95.9 by patches, 99.6
     // without; 2 M 251 and 259; 3.4 M 451 and 449, in 64 instances with 18.8 M particles 622 and 610).
     constexpr int PATCH_MAX_F = 2500000;
@@ -444,7 +444,8 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
         } catch (const std::bad_alloc &) {
             return FETDPIC_ENOMEM;
         }
-        ctx->patches = ps.ok && field_smem(f32, ps.max_r, ps.max_e) <= FIELD_SMEM_MAX;
+        ctx->patches = ps.ok && field_smem(f32, ps.max_r, ps.max_e) <= FIELD_SMEM_MAX &&
+                       patches_pay(ps, ctx->E, (long long)mci.size());
     }
     // else sliced ELL over all rows (32 rows per slice, column-major inside a slice)
     std::vector<long long> soff(1, 0);

@@ -104,6 +104,9 @@ struct PatchInput {
 PatchSet build_patches(const PatchInput &in, int T);
 // Triangles of a patch on a mesh of F triangles.
 int field_patch_size(int F, int sms);
+// Whether the update by patches is worth what it computes twice, on a mesh of `edges` edges and an
+// inverse of `entries` entries.
+bool patches_pay(const PatchSet &S, long long edges, long long entries);
 // Shared memory of one block; a context whose patches need more uses launch_ampere.
 size_t field_smem(bool f32, int max_r, int max_e);
 constexpr size_t FIELD_SMEM_MAX = 100 * 1024;

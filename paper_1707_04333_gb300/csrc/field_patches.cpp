@@ -119,6 +119,22 @@ int field_patch_size(int F, int sms)
     return (int)(T < least ? least : T);
 }
 
+// The patches recompute the curl on the edges around them and the rows of the
+// ring, and pad the rows in slices of their own.  On a mesh whose storage order
+// is compact that is little (the weighted sum below stays under 0.7 of the
+// bound, also with small patches and high levels of the inverse, and the patches
+// win throughout: 28,800 triangles, level 6, 12.9 us a step against 19.7).  Where it
+// is not (many triangles in one cell of the curve, in no order), the separate
+// kernels win, the sooner the larger the mesh.  Patches and separate kernels, us
+// a step, by the weighted sum over the bound: 8,192 triangles, 0.80: 10.4 and
+// 11.3; 20,000, 0.98: 10.7 and 11.4, 1.66: 14.8 and 11.5; 51,200, 1.07: 14.5 and
+// 15.6, 1.88: 18.1 and 16.0; 200,978, 0.61: 20.8 and 24.0, 1.47: 31.9 and 24.9.
+bool patches_pay(const PatchSet &S, long long edges, long long entries)
+{
+    const double extra = 4.0 * (double)S.xlist.size() + (double)S.val.size() - (double)entries;
+    return extra <= 9e5 + 0.85 * (double)(edges + entries);
+}
+
 size_t field_smem(bool f32, int max_r, int max_e)
 {
     return sizeof(double) * ((size_t)max_r + max_e) + (f32 ? sizeof(float) * (size_t)max_r : 0);

@@ -34,7 +34,7 @@ static bool make(Input &I, int nx, int ny, int level, bool scattered)
 {
     std::mt19937 g(3);
     std::uniform_real_distribution<double> U(-0.2, 0.2);
-    const double h = scattered ? 1e-7 : 1.0;
+    const double h = scattered ? 1e-11 : 1.0;
     std::vector<double> xy;
     std::vector<int> t;
     for (int j = 0; j <= ny; ++j)
@@ -133,6 +133,15 @@ int main()
             const char *bad = S.ok ? check(I, S) : "no tables";
             if (bad) { printf("%d x %d, level %d, T %d: %s\n", s.nx, s.ny, s.level, T, bad); return 1; }
         }
+    }
+    // worth their while on compact meshes of any level, not on large ones in no order
+    struct { int nx, ny, level; bool scattered, pay; } uses[] = {{1, 1, 1, false, true}, {60, 3, 3, false, true}, {90, 80, 1, false, true}, {120, 120, 2, false, true},
+                                                                 {50, 50, 6, false, true}, {20, 20, 2, true, true}, {160, 160, 2, true, false}, {64, 64, 4, true, false}};
+    for (auto &u : uses) {
+        Input I;
+        if (!make(I, u.nx, u.ny, u.level, u.scattered)) return 1;
+        const PatchSet S = build_patches(I.in(), field_patch_size(I.M.nf, 152));
+        if (patches_pay(S, I.M.ne, (long long)I.mci.size()) != u.pay) { printf("%d x %d, level %d: pay\n", u.nx, u.ny, u.level); return 1; }
     }
     // an allocation that fails, in a thread or not, arrives as an exception
     Input I;

@@ -55,3 +55,38 @@ def test_contexts_with_large_patches_live_together(precision, graphs):
         whole.close()
     for s in sims:
         s.close()
+
+
+def _clustered(nx, level, side=112):
+    """The square in no order of nx x nx cells beside an ordinary one: the patches pay on the whole, and
+    those of the cluster are large."""
+    w = _scattered(nx, nx)
+    m = inputs.jittered_delaunay(side, side, 1.0, 1.0, 0.2, seed=7)
+    n = len(w.mesh.nodes)
+    nodes = np.concatenate([w.mesh.nodes, m.nodes + 1.5])
+    w.mesh = inputs.Mesh(nodes, np.concatenate([w.mesh.triangles, m.triangles + n]).astype(np.int32), 3.0, 3.0)
+    return w
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+def test_large_patches_among_small_ones(graphs):
+    """55 and 50 KB a block (host build of the tables); the first context steps after the second exists."""
+    from paper_1707_04333_gb300 import fetdpic
+
+    def sim(level, whole=False):
+        return fetdpic.Simulation(_clustered(42, level), precision="fp32", spai_level=level, sort_interval=-1,
+                                  use_graphs=graphs and not whole, fuse_field_update=whole).load()
+    sims = [sim(7), sim(6)]
+    for s, level in zip(sims, (7, 6)):
+        whole = sim(level, True)
+        s.step(1, "boris").sync()
+        whole.step(1, "boris").sync()
+        fetdpic.fetdpic_stage_times(s.h)
+        s.step(8, "boris").sync()
+        whole.step(8, "boris").sync()
+        # Faraday, then particles and one field launch a step: the patches are in use
+        assert fetdpic.fetdpic_stage_times(s.h)[1] == 17
+        assert _equal(s, whole)
+        whole.close()
+    for s in sims:
+        s.close()
