@@ -392,7 +392,8 @@ int fetdpic_read_edges(fetdpic_ctx *ctx, int inst, int *edges);
 int fetdpic_read_spai(fetdpic_ctx *ctx, int inst, long long *rowptr, int *row_edge, int *col, double *val);
 
 /* Autotuner (no counterpart in the paper, which reports no kernels): times
- * short trials of every (FP32 particle-kernel variant in {2, ..., 12}) x (sort
+ * short trials of every (FP32 particle-kernel variant, 0 where the default
+ * is a pair of kernels without a number of its own) x (sort
  * interval in {8, 12, 16, 32}) combination -- only the sort interval for FP64,
  * nothing if sorting is off -- starting each from the current state, keeps
  * the fastest per step (sort cost included), and restores the particle and

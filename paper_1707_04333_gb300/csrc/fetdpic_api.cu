@@ -977,10 +977,11 @@ static constexpr Hybrid HYBRIDS[] = {{17, 12, 14, 6}, {18, 12, 14, 4}, {21, 19, 
 //     does not pay (two per triangle: 42.5 with variant 12, 44.7 with 22; eight: 18.7 against 20.1).
 //     Counted where the particles are, since a batch may be uneven (16 instances with 2 to 96 per
 //     triangle, 6.8 in all but 30 around the mean particle: 53.9 with the window kernels, 56.6 without);
-//   - else an early and a late kernel.  Early, 28 warps per SM for the Vay pusher, 24 for the others,
-//     whose kernels spill at 72 registers (8 M particles, Higuera-Cary: 130.5 against 134.3).  Late, the 20-warp window kernel up to 2 M particles,
-//     where its few more particles per warp cost less than registers held back from it (1.1 M in 16
-//     instances: 53.8 against 55.6), the 24-warp one above (8 M: 130.2 against 131.3).
+//   - else an early and a late kernel.  Early, 28 warps per SM for the Vay pusher, 24 for the others, whose
+//     28-warp kernels spill: 6.25 M particles above gamma = 10 161.6 against 168.7 (Higuera-Cary) and 152.6
+//     against 159.3 (Boris), 8 M thermal ones 130.9 against 129.9 and 129.4 against 128.3.  Late, the 20-warp
+//     window kernel up to 2 M particles, where its few more particles per warp cost less than registers held
+//     back from it (1.1 M in 16 instances: 53.8 against 55.6), the 24-warp one above (8 M: 130.2 against 131.3).
 static Hybrid kernels_of(const fetdpic_ctx *ctx, int pusher)
 {
     const int v = ctx->p.kernel_variant;
@@ -1960,6 +1961,15 @@ extern "C" int fetdpic_autotune(fetdpic_ctx *ctx, int pusher, int trial_steps, i
     rc = copy_state(true);
     std::vector<int> variants = ctx->p.precision == FETDPIC_FP32 ? std::vector<int>{2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 14, 17, 18, 19, 20, 21, 22}
                                                           : std::vector<int>{3};
+    // the default where it is none of them (above 2 M particles with 12 or more per triangle, the pushers
+    // other than Vay: variant 12, then 20)
+    if (ctx->p.precision == FETDPIC_FP32) {
+        ctx->p.kernel_variant = 0;
+        const Hybrid d = kernels_of(ctx, pusher);
+        bool listed = d.early == d.late;
+        for (const Hybrid &h : HYBRIDS) listed = listed || (h.early == d.early && h.late == d.late && h.steps == d.steps);
+        if (!listed) variants.push_back(0);
+    }
     std::vector<int> sorts = keep_sort < 0 ? std::vector<int>{-1} : std::vector<int>{8, 12, 16, 32};
     double best = 1e300;
     int bv = keep_variant, bs = keep_sort;
