@@ -806,7 +806,9 @@ static int finalize(fetdpic_ctx *ctx)
         D.alpha = S.q * dt / (2.0 * S.m);
         const double qr = qref[S.inst] > 0 ? qref[S.inst] : 1.0;
         D.wfix = (S.q / qr) * ctx->fixscale[S.inst];
-        D.qfix = D.wfix;
+        // (below 1e-250 of a unit every particle's charge rounds to 0; k_charge32's integer product needs the
+        // factor to leave it in range)
+        D.qfix = std::fabs(D.wfix) < 1e-250 ? 0.0 : D.wfix;
         D.wfix32 = (float)D.wfix;
         D.dt = dt; D.c = P.c; D.ic2 = 1.0 / (P.c * P.c);
         D.ext_ex = I.ext_ex; D.ext_ey = I.ext_ey; D.ext_bz = I.ext_bz;
