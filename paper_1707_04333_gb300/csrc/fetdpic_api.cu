@@ -257,6 +257,7 @@ static int take_status(fetdpic_ctx *ctx)
     CK(cudaMemcpyAsync(st, ctx->status, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     const unsigned s = *st;
+    if (s) CK(cudaSetDevice(ctx->device));      // a clear needs the stream's device
     if (s) CK(cudaMemsetAsync(ctx->status, 0, sizeof(unsigned), ctx->stream));
     // a step that timed out is incomplete: drop the current it deposited, and the counts a grid
     // barrier that gave up left behind
@@ -1725,6 +1726,7 @@ extern "C" int fetdpic_check(fetdpic_ctx *ctx, int inst, double *dce_max, double
 {
     if (!ctx || inst < 0 || inst >= (int)ctx->mesh.size()) return FETDPIC_EINVAL;
     if (!ctx->chk_out) return ctx->fail(FETDPIC_ESTATE, "check_interval is 0: no checks are computed");
+    CK(cudaSetDevice(ctx->device));
     CK(cudaStreamSynchronize(ctx->stream));
     double v[3] = {0, 0, 0};
     CK(cudaMemcpy(v, ctx->chk_out + 3 * inst, sizeof(v), cudaMemcpyDeviceToHost));
