@@ -761,7 +761,7 @@ static void reset_gauss_reference(fetdpic_ctx *ctx)
 static bool soft_constant(double v)
 {
     const double m = std::fabs(v);
-    return m == 0.0 || (m >= 0x1p-100 && m < 0x1p64);
+    return (m == 0.0) | ((m >= 0x1p-100) & (m < 0x1p64));
 }
 
 // Move the staged species to the device: padded species ranges, block ->
@@ -834,13 +834,15 @@ static int finalize(fetdpic_ctx *ctx)
         for (int k = 0; k < ni; ++k) { all += n[k]; sum += n[k] * (n[k] / ctx->mesh[k].nf); }
         ctx->density = all > 0.0 ? sum / all : 0.0;
     }
-    ctx->soft64 = true;
-    for (const Species &D : ctx->sp)
-        ctx->soft64 = ctx->soft64 && soft_constant(D.alpha) && soft_constant(D.ic2) && soft_constant(D.dt) &&
-                      soft_constant(D.wfix);
-    for (const HostMesh &M : ctx->mesh)
-        for (const std::vector<double> *g : {&M.gx, &M.gy, &M.X, &M.Y})
-            ctx->soft64 = ctx->soft64 && std::all_of(g->begin(), g->end(), soft_constant);
+    if (P.precision == FETDPIC_FP64) {           // the FP32 path does not ask
+        bool soft = true;
+        for (const Species &D : ctx->sp)
+            soft = soft && soft_constant(D.alpha) && soft_constant(D.ic2) && soft_constant(D.dt) && soft_constant(D.wfix);
+        for (const HostMesh &M : ctx->mesh)
+            for (const std::vector<double> *g : {&M.gx, &M.gy, &M.X, &M.Y})
+                for (const double v : *g) soft &= soft_constant(v);     // no branch: one pass of vector code
+        ctx->soft64 = soft;
+    }
     ctx->P = off;
     ctx->nblocks = off / ctx->block;
     if (off >= (1ll << 31))      // particle slots and load indices are 32-bit
