@@ -129,7 +129,8 @@ struct fetdpic_ctx {
     void *xfer = nullptr; size_t xfer_bytes = 0;
     // page-locked host memory: small reads come back in one copy each, with the status word behind
     // them, and one wait (SMALL_READ bytes for them, then the status)
-    char *pin = nullptr;
+    char *pin = nullptr, *pin_locked = nullptr;
+    std::vector<char> pin_plain;              // in its place where the host has none to lock
     // asynchronous particle reads: staging of their own (one region per species), copied to the
     // host on the io stream while the context stream goes on; set up by the first such read
     cudaStream_t io = nullptr;
@@ -171,7 +172,7 @@ struct fetdpic_ctx {
             if (p.dev_free) p.dev_free(q, p.alloc_user);
             else cudaFree(q);
         }
-        if (pin) cudaFreeHost(pin);
+        if (pin_locked) cudaFreeHost(pin_locked);
         for (auto &x : ev) cudaEventDestroy(x);
         for (auto &x : ev_rd_done) if (x) cudaEventDestroy(x);
         if (ev_rd) cudaEventDestroy(ev_rd);
@@ -298,11 +299,13 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
     CK(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
 
-    if (cudaHostAlloc((void **)&ctx->pin, SMALL_READ + 256, cudaHostAllocDefault) != cudaSuccess) {
-        ctx->pin = nullptr;
+    if (cudaHostAlloc((void **)&ctx->pin_locked, SMALL_READ + 256, cudaHostAllocDefault) != cudaSuccess) {
+        // no page-locked memory to be had: reads go through ordinary memory, slower
+        ctx->pin_locked = nullptr;
         cudaGetLastError();
-        return FETDPIC_ENOMEM;
+        try { ctx->pin_plain.resize(SMALL_READ + 256); } catch (const std::bad_alloc &) { return FETDPIC_ENOMEM; }
     }
+    ctx->pin = ctx->pin_locked ? ctx->pin_locked : ctx->pin_plain.data();
 
     // ---- host setup per instance
     ctx->mesh.resize(n_inst);
