@@ -87,14 +87,14 @@ typedef enum {
      * positions and momenta (Boris-tan excepted: tan is not correctly rounded). */
     FETDPIC_FP64 = 0,
     /* FP32 gather/push/deposit with cell-local barycentric positions and
-     * momenta in units of c; for particles with gamma > 10 the Lorentz factor
-     * and momentum update in two and three floats, whose error against
-     * extended precision is below that of the same push in FP64 with Newton
-     * roots, or in FP64 (gamma above 3.1e8; a kick or |q B dt / 2m| above
-     * gamma / 8, gamma / 31 for Boris-tan); FP64 for the field unknowns e, b, the Faraday update, C^T [*mu^-1] b - i
-     * and the checks.  The SPAI product dt M r of
-     * the Ampere update runs in FP32 (FP32 matrix values, r rounded to FP32,
-     * FP32 sums) and is added to the FP64 e. */
+     * momenta in units of c.  The Lorentz factor and momentum update of
+     * particles with gamma > 10 run in two and three floats, with an error
+     * against extended precision below that of the same push in FP64 with
+     * Newton roots; in FP64 above gamma = 3.1e8 and where the kick or
+     * |q B dt / 2m| is above gamma / 8 (gamma / 31 for Boris-tan).  FP64 for
+     * the field unknowns e, b, the Faraday update, C^T [*mu^-1] b - i and the
+     * checks.  The SPAI product dt M r of the Ampere update runs in FP32 (FP32
+     * matrix values, r rounded to FP32, FP32 sums) and is added to the FP64 e. */
     FETDPIC_FP32 = 1
 } fetdpic_precision;
 

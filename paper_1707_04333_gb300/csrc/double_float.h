@@ -22,8 +22,9 @@
 //   gamma 10 to 1000, kick and |beta| between gamma / 33 and gamma / 8
 //     Higuera-Cary  u 6.1e-16 (7.0e-15) / 5.0e-16 (5.3e-15)   Vay        2.2e-15 (8.3e-15) / 4.5e-16 (5.2e-15)
 //     Boris         u 6.6e-16 (8.1e-15) / 4.5e-16 (4.1e-15)   Boris-tan  1.8e-16 (2.0e-15) / 1.2e-16 (1.3e-15)
-// and below the FP64 push's likewise over gamma 10 to 3e8 and kicks down to 1e-9 gamma.  The stored FP32 momenta and the FP32
-// velocities, rounded at 6e-8, agree but for one in a million.
+// and below the FP64 push's likewise over gamma 10 to 3e8 and kicks down to
+// 1e-9 gamma.  The stored FP32 momenta and the FP32 velocities, rounded at 6e-8,
+// agree but for one in a million.
 //
 // Host code runs the same functions (tests/double_float_host.cpp measures them).
 #pragma once

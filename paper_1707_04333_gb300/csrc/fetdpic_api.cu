@@ -432,12 +432,14 @@ extern "C" int fetdpic_create(fetdpic_ctx **out, const fetdpic_params *prm, int 
     ctx->nfree = (long long)mrow.size();
     const bool f32 = P.precision == FETDPIC_FP32;
     // the field update by patches, unless the cooperative form is asked for, a patch's edges do not fit
-    // its block (a dense inverse) or the patches would compute too much twice.  Beyond PATCH_MAX_F triangles the update is bound by memory
-    // bandwidth, of which the three kernels need less (us a step: 0.72 M triangles 95.9 by patches, 99.6
-    // without; 2 M 251 and 259; 3.4 M 451 and 449, in 64 instances with 18.8 M particles 622 and 610).
-    constexpr int PATCH_MAX_F = 2500000;
+    // its block (a dense inverse) or the patches would compute too much twice.  Beyond patch_max
+    // triangles the update is bound by memory bandwidth, of which the three kernels need less.  Us a step
+    // by patches and without, FP32: 0.98 M triangles 98.6 and 99.3, 1.45 M 138.4 and 140.2 (with 2.9 M
+    // particles 181.7 and 184.0), 1.69 M 162.8 and 161.5 (219.4 and 218.3), 2 M 194.7 and 188.4; FP64:
+    // 0.64 M 127.1 and 130.1, 0.82 M 153.0 and 152.5, 0.98 M 180.6 and 178.7, 1.69 M 284.8 and 277.4.
+    const int patch_max = f32 ? 1550000 : 750000;
     PatchSet ps;
-    if (!P.fuse_field_update && P.spai_level >= 0 && ctx->F <= PATCH_MAX_F) {
+    if (!P.fuse_field_update && P.spai_level >= 0 && ctx->F <= patch_max) {
         std::vector<int> te(3 * (size_t)ctx->F), row(ctx->E, -1);
         for (int f = 0; f < ctx->F; ++f)
             for (int m = 0; m < 3; ++m) te[3 * (size_t)f + m] = tp[f].ew[m] >> 1;
@@ -981,15 +983,19 @@ static constexpr Hybrid HYBRIDS[] = {{17, 12, 14, 6}, {18, 12, 14, 4}, {21, 19, 
 //   - up to one 64-particle chunk per SM: the kernel with one particle per lane is through it soonest
 //     (64 particles: 6.15 against 6.7 with variant 22; 4,000: 7.0 against 7.6; with two chunks per
 //     SM variant 12 is ahead, 8.72 against 8.93);
-//   - fewer than twelve particles per triangle: runs are short from the start and the window's flush
-//     does not pay (two per triangle: 42.5 with variant 12, 44.7 with 22; eight: 18.7 against 20.1).
-//     Counted where the particles are, since a batch may be uneven (16 instances with 2 to 96 per
-//     triangle, 6.8 in all but 30 around the mean particle: 53.9 with the window kernels, 56.6 without);
+//   - fewer than twenty particles per triangle: runs are short and the window's flush does not pay.
+//     Variant 12 against window kernels (Vay): 8,192 triangles 4 to 30 a triangle 2 to 5 % ahead
+//     throughout; 51,200 triangles 4 a triangle 14.3 and 15.8, 8 16.5 and 17.9, 10 18.6 and 18.0, 12 18.8
+//     and 20.1, 14 21.0 and 20.2, 16 21.5 and 22.5, 20 23.8 and 24.0; 180,000 triangles 10 a triangle 42.2
+//     and 43.8, 16 57.2 and 57.4, 20 65.8 and 66.6; 201k, 40 a triangle 131.6 and 128.9.  Counted
+//     where the particles are, since a batch may be uneven (16 instances with 2 to 96 per triangle, 6.8 in
+//     all but 30 around the mean particle: 53.9 with the window kernels, 56.6 without);
 //   - else an early and a late kernel.  Early, 28 warps per SM for the Vay pusher, 24 for the others, whose
 //     28-warp kernels spill: 6.25 M particles above gamma = 10 161.6 against 168.7 (Higuera-Cary) and 152.6
 //     against 159.3 (Boris), 8 M thermal ones 130.9 against 129.9 and 129.4 against 128.3.  Late, the 20-warp
-//     window kernel up to 2 M particles, where its few more particles per warp cost less than registers held
-//     back from it (1.1 M in 16 instances: 53.8 against 55.6), the 24-warp one above (8 M: 130.2 against 131.3).
+//     window kernel up to 2 M particles (1.1 M in 16 instances: 53.8 against 55.6), the 24-warp one above:
+//     they are within 1.3 % of one another from 0.8 to 3.9 M, 5.8 M take 89.2 with the 24-warp one and 109.8
+//     with the other.
 static Hybrid kernels_of(const fetdpic_ctx *ctx, int pusher)
 {
     const int v = ctx->p.kernel_variant;
@@ -998,7 +1004,7 @@ static Hybrid kernels_of(const fetdpic_ctx *ctx, int pusher)
     if (v != 0) return Hybrid{v, v, v, 0};
     const long long n64 = ctx->P / 64;
     if (n64 <= ctx->sms) return Hybrid{0, 4, 4, 0};
-    if (ctx->density < 12.0) return Hybrid{0, 12, 12, 0};
+    if (ctx->density < 20.0) return Hybrid{0, 12, 12, 0};
     return Hybrid{0, pusher == FETDPIC_VAY ? 19 : 12, n64 < 32768 ? 14 : 20, 6};
 }
 
@@ -1970,7 +1976,7 @@ extern "C" int fetdpic_autotune(fetdpic_ctx *ctx, int pusher, int trial_steps, i
     rc = copy_state(true);
     std::vector<int> variants = ctx->p.precision == FETDPIC_FP32 ? std::vector<int>{2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 14, 17, 18, 19, 20, 21, 22}
                                                           : std::vector<int>{3};
-    // the default where it is none of them (above 2 M particles with 12 or more per triangle, the pushers
+    // the default where it is none of them (above 2 M particles with 20 or more per triangle, the pushers
     // other than Vay: variant 12, then 20)
     if (ctx->p.precision == FETDPIC_FP32) {
         ctx->p.kernel_variant = 0;

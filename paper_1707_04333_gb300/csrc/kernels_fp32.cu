@@ -776,9 +776,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_particles32x2(StepArgs32 a)
         dw.nt = tc >= 0 ? WT : 0;
         __syncthreads();
     }
-    // Only the field records come from the kernel this one may overlap (Faraday); the
-    // particle state and the cleared current were written before Faraday started, so the
-    // first state load and the window set-up go ahead of the wait.
+    // Ahead of the wait only the particle state may be read (the first state load and the window
+    // set-up): the field records and the cleared current both come from the kernel this one may
+    // overlap (Faraday, or the field update that carries it), so no gather and no deposit before it.
     pdl_begin();
     if (c < cend) {
         for (; c < cend; ++c) {
