@@ -103,12 +103,13 @@ void build_range(PatchSet &S, const PatchInput &in, const std::vector<int> &own,
 // 44.6 in one wave, 49.8 in one and a half).  One wave as long as its patches
 // are of at most 850 triangles, then two: 231,200 triangles 30.7 in one and 33.0
 // in two, 312,050 42.4 and 45.8, 364,658 49.6 and 52.6, 387,200 (patches of 850)
-// 51.8 and 54.0, 410,418 (901) 57.2 and 56.3, 428,738 (941) 68.1 and 58.7: there
-// three blocks' tables pass 100 KB, and the SM sets a third more of its L1
-// aside for shared memory.  Two and three waves differ alike (720,000 triangles
-// 91.9 and 97.8; 768,800, patches of 843, 96.3 and 101.1).  At least 64
-// triangles: smaller patches gain nothing on 2,048 triangles (6.77 with 48, 6.71
-// with 64, 6.88 with 96).
+// 51.8 and 54.0, 410,418 (901) 57.2 and 56.3, 428,738 (941) 68.1 and 58.7.  The
+// turn lies in the overlap with the particle kernels around it, not in the
+// kernel: alone and cold it takes 39.0 us in one wave there and 43.5 in two, and
+// no setting of the SM's shared memory moves it.  Two and three waves differ
+// alike (720,000 triangles 91.9 and 97.8; 768,800, patches of 843, 96.3 and
+// 101.1).  At least 64 triangles: smaller patches gain nothing on 2,048 triangles
+// (6.77 with 48, 6.71 with 64, 6.88 with 96).
 int field_patch_size(int F, int sms)
 {
     constexpr int most = 850, least = 64;

@@ -13,10 +13,11 @@
 //
 // Measured (device time of a step, graph replay, with the particles): 2,048
 // triangles and 64 electrons 9.8 -> 6.6 us, 8,192 triangles and 328k particles
-// 19.0 -> 15.6, 320k triangles and 640k particles 52.7 -> 44.5, 201k triangles
-// and 8 M particles 134.8 -> 129.  Bound by the latency of the loads between
-// its phases and, on the large meshes, by the FP64 pipe (2 lanes per SM and
-// clock: conversions to and from FP32 run in integer arithmetic beside it).
+// 19.0 -> 15.6, 320k triangles and 640k particles 52.7 -> 42.8, 201k triangles
+// and 8 M particles 134.8 -> 128.9.  Bound by the FP64 pipe (2 lanes per SM and
+// clock, 53 % busy; conversions to and from FP32 run in integer arithmetic beside
+// it) and by the latency of the loads between its phases (320k triangles: 26 of
+// a warp's 36 cycles per issue wait for memory or a barrier, issue 27 %, DRAM 37 %).
 #include <cuda_runtime.h>
 
 #include "fetdpic_internal.h"
