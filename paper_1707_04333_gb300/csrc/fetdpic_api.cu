@@ -845,7 +845,7 @@ static int finalize(fetdpic_ctx *ctx)
             soft = soft && soft_constant(D.alpha) && soft_constant(D.ic2) && soft_constant(D.dt) && soft_constant(D.wfix);
         for (const HostMesh &M : ctx->mesh)
             for (const std::vector<double> *g : {&M.gx, &M.gy, &M.X, &M.Y})
-                for (const double v : *g) soft &= soft_constant(v);     // no branch: one pass of vector code
+                for (const double v : *g) soft &= soft_constant(v);
         ctx->soft64 = soft;
     }
     ctx->P = off;
@@ -984,12 +984,13 @@ static constexpr Hybrid HYBRIDS[] = {{17, 12, 14, 6}, {18, 12, 14, 4}, {21, 19, 
 //     (64 particles: 6.15 against 6.7 with variant 22; 4,000: 7.0 against 7.6; with two chunks per
 //     SM variant 12 is ahead, 8.72 against 8.93);
 //   - fewer than twenty particles per triangle: runs are short and the window's flush does not pay.
-//     Variant 12 against window kernels (Vay): 8,192 triangles 4 to 30 a triangle 2 to 5 % ahead
-//     throughout; 51,200 triangles 4 a triangle 14.3 and 15.8, 8 16.5 and 17.9, 10 18.6 and 18.0, 12 18.8
-//     and 20.1, 14 21.0 and 20.2, 16 21.5 and 22.5, 20 23.8 and 24.0; 180,000 triangles 10 a triangle 42.2
-//     and 43.8, 16 57.2 and 57.4, 20 65.8 and 66.6; 201k, 40 a triangle 131.6 and 128.9.  Counted
-//     where the particles are, since a batch may be uneven (16 instances with 2 to 96 per triangle, 6.8 in
-//     all but 30 around the mean particle: 53.9 with the window kernels, 56.6 without);
+//     Variant 12 against window kernels (Vay): 8,192 triangles, 4 to 30 a triangle, 1.5 to 6 % ahead
+//     throughout; 20,000 2 to 12 % ahead but at 12 and 24 a triangle (2 to 3 % behind); 51,200, 4 a
+//     triangle 14.3 and 15.8, 8 16.5 and 17.9, 10 18.6 and 18.0, 12 18.8 and 20.1, 14 21.0 and 20.2, 16 21.5
+//     and 22.5, 20 23.8 and 24.0; 180,000, 10 a triangle 42.2 and 43.8, 16 57.2 and 57.4, 20 65.8 and 66.6;
+//     201k, 40 a triangle 131.6 and 128.9.  Counted where the particles are, since a batch may be uneven
+//     (16 instances with 2 to 96 per triangle, 6.8 in all but 30 around the mean particle: 53.9 with the
+//     window kernels, 56.6 without);
 //   - else an early and a late kernel.  Early, 28 warps per SM for the Vay pusher, 24 for the others, whose
 //     28-warp kernels spill: 6.25 M particles above gamma = 10 161.6 against 168.7 (Higuera-Cary) and 152.6
 //     against 159.3 (Boris), 8 M thermal ones 130.9 against 129.9 and 129.4 against 128.3.  Late, the 20-warp
