@@ -150,8 +150,8 @@ typedef struct {
                                 grid barrier with a bounded wait (FETDPIC_ETIMEOUT if it gives
                                 up); 0 = one launch of independent mesh patches, which inside a
                                 call carries the next step's Faraday update too, or two launches
-                                where the patches do not fit shared memory (the default: faster
-                                on GB300).  Same arithmetic, same results. */
+                                where the patches do not fit shared memory or do not pay (large or
+                                scattered meshes) (the default: faster on GB300).  Same arithmetic, same results. */
 } fetdpic_params;
 
 /* One simulation instance (mesh + fields).  Instances share nothing but the
